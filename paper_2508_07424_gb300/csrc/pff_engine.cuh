@@ -675,7 +675,7 @@ inline void pinv_solve(int m, const double *Min, const double *b, double rcond, 
 // Column-tile table of the autotuner: process-wide, backed by a text cache file of lines
 // "<key> <cw_y> <cw_z>" (the last line for a key wins).
 // ------------------------------------------------------------------------------------------------
-constexpr int kColumnPassRev = 2;  // 16 points per lane on lines of 16-128 points
+constexpr int kColumnPassRev = 3;  // transposing transforms, FP64 lines in fixed point
 inline std::mutex g_tile_mu;
 inline std::mutex g_tune_mu;  // one measurement at a time, so concurrent handles do not skew it
 inline std::map<std::string, std::pair<int, int>> g_tiles;
@@ -797,7 +797,7 @@ struct Engine : EngineBase {
     T *dr = nullptr, *dz = nullptr, *dp = nullptr, *dq = nullptr;
     double *eps_it = nullptr, *eps_com = nullptr, *xh = nullptr, *gh = nullptr, *dtmp = nullptr;
     C *spec = nullptr;
-    std::map<int, C *> tw;
+    std::map<int, line_w<T> *> tw;
     Scal *sc = nullptr, *sc2 = nullptr, *h_sc = nullptr, *sc3 = nullptr;
     double *partials = nullptr;
     int G = 0;
@@ -941,6 +941,15 @@ struct Engine : EngineBase {
         return (P *)p;
     }
 
+    // Twiddle table of a line of L points for transforms in precision U.
+    template <typename U> line_w<U> *twiddles(int L) {
+        std::vector<line_w<U>> h(L);
+        for (int m = 0; m < L; ++m) axis_twiddle(m, L, h[m]);
+        auto *d = alloc<line_w<U>>(L);
+        CK(cudaMemcpyAsync(d, h.data(), L * sizeof(h[0]), cudaMemcpyHostToDevice, st));
+        return d;
+    }
+
     explicit Engine(const rve_config &c) {
         cfg = c;
         if (kSingle) {
@@ -972,7 +981,7 @@ struct Engine : EngineBase {
         if (const char *aws = std::getenv("PFF_AXIS_WARPS")) aw = std::max(1, std::min(16, std::atoi(aws)));
         if (c.stream) st = (cudaStream_t)c.stream;
         else { CK(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking)); own_stream = true; }
-        CK(axis_twiddles_init());  // constant-bank twiddles of the column passes (this device)
+        CK(axis_twiddles_init());  // constant-bank twiddles of the FP32 column passes (this device)
         try {
             gid = alloc<int>(N); gid0 = alloc<int>(N);
             phi = alloc<T>(N); phi_trial = alloc<T>(N); phi_cur = alloc<T>(N); H = alloc<T>(N); Hcur = alloc<T>(N);
@@ -989,15 +998,7 @@ struct Engine : EngineBase {
             CK(cudaMallocHost(&h_sc, sizeof(Scal)));
             for (int L : {g.nx, g.ny, g.nz}) {
                 if (L < 4 || tw.count(L)) continue;
-                std::vector<C> h(L);
-                for (int m2 = 0; m2 < L; ++m2) {
-                    long double a = -2.0L * 3.14159265358979323846264338327950288L * (long double)m2 / (long double)L;
-                    h[m2].x = (T)std::cos(a);
-                    h[m2].y = (T)std::sin(a);
-                }
-                C *d = alloc<C>(L);
-                CK(cudaMemcpyAsync(d, h.data(), L * sizeof(C), cudaMemcpyHostToDevice, st));
-                tw[L] = d;
+                tw[L] = twiddles<T>(L);
             }
             // frequency tables xi~ = 2 pi k / n with the Nyquist frequency set to zero
             auto xi_host = [](int n, int len, bool half) {
@@ -1059,7 +1060,7 @@ struct Engine : EngineBase {
         for (int cw = 1; cw <= 16; cw *= 2) {
             int th;
             size_t sm;
-            axis_shape<C>(L, NM, cw, th, sm);
+            axis_shape<T>(L, NM, cw, th, sm);
             if (sm <= 200 * 1024) v.push_back(cw);
         }
         if (v.empty()) v.push_back(1);
@@ -1211,13 +1212,13 @@ struct Engine : EngineBase {
     // residual passes of the iterative refinement (allocated on first use).
     typedef typename cplx_of<double>::type C64;
     C64 *spec64 = nullptr;
-    std::map<int, C64 *> tw64;
+    std::map<int, line_w<double> *> tw64;
     double *xi64_x = nullptr, *xi64_y = nullptr, *xi64_z = nullptr;
     template <typename U> typename cplx_of<U>::type *spec_of() {
         if constexpr (std::is_same<U, T>::value) return spec;
         else return spec64;
     }
-    template <typename U> const typename cplx_of<U>::type *tw_of(int L) {
+    template <typename U> const line_w<U> *tw_of(int L) {
         if constexpr (std::is_same<U, T>::value) return tw[L];
         else return tw64[L];
     }
@@ -1227,15 +1228,7 @@ struct Engine : EngineBase {
         spec64 = alloc<C64>((size_t)std::max(NS, D) * (size_t)(((g.nx / 2 + 1 + 15) / 16) * 16) * g.ny * g.nz);
         for (int L : {g.nx, g.ny, g.nz}) {
             if (L < 4 || tw64.count(L)) continue;
-            std::vector<C64> h(L);
-            for (int m2 = 0; m2 < L; ++m2) {
-                long double a = -2.0L * 3.14159265358979323846264338327950288L * (long double)m2 / (long double)L;
-                h[m2].x = (double)std::cos(a);
-                h[m2].y = (double)std::sin(a);
-            }
-            C64 *d = alloc<C64>(L);
-            CK(cudaMemcpyAsync(d, h.data(), L * sizeof(C64), cudaMemcpyHostToDevice, st));
-            tw64[L] = d;
+            tw64[L] = twiddles<double>(L);
         }
         auto xi_host = [](int n, int len, bool half) {
             std::vector<double> v(len, 0.0);
@@ -1256,44 +1249,39 @@ struct Engine : EngineBase {
         xi64_y = up(xi_host(g.ny, g.ny, false));
         xi64_z = up(xi_host(g.nz, g.nz, false));
     }
-    template <typename U = T> void xcfg(int &threads, int &blocks, size_t &smem1) const {
-        const int TL = g.nx / 4;
-        const long long pairs = (long long)g.ny * g.nz / 2;
-        int RP = std::max(1, 128 / TL);
-        if (RP > pairs) RP = (int)pairs;
-        threads = RP * TL;
-        blocks = (int)(pairs / RP);
-        smem1 = (size_t)RP * g.nx * sizeof(typename cplx_of<U>::type);
-    }
+    template <typename U = T> XShape xshape() const { return x_shape<U>(g.nx, (long long)g.ny * g.nz / 2); }
     template <int NC, class Pro, typename U = T> void x_fwd(const Pro &pro, Scal *s) {
-        int th, bl; size_t sm; xcfg<U>(th, bl, sm);
+        const XShape x = xshape<U>();
+        const size_t sm = x_smem<U>(g.nx, x.RP, NC);
         auto k = k_x_fwd<U, NC, Pro>;
-        prep_x(k, sm * NC);
+        prep_x(k, sm);
         cudaEvent_t e = tbeg(std::is_same<U, T>::value ? 2 : 7, is_cg_dir<Pro>::value ? 2 : 0,
                              xbytes<U>(NC, rw_words<Pro>()), xflops(NC));
-        k<<<bl, th, sm * NC, st>>>(g, pro, spec_of<U>(), tw_of<U>(g.nx), partials, s);
+        k<<<x.blocks, x.threads, sm, st>>>(g, x.RP, pro, spec_of<U>(), tw_of<U>(g.nx), partials, s);
         CK(cudaGetLastError());
         tend(e);
         ++launches;
     }
     template <int NC, class Epi, typename U = T> void x_inv(const Epi &epi, Scal *s) {
-        int th, bl; size_t sm; xcfg<U>(th, bl, sm);
+        const XShape x = xshape<U>();
+        const size_t sm = x_smem<U>(g.nx, x.RP, NC);
         auto k = k_x_inv<U, NC, Epi>;
-        prep_smem(k, sm * NC);
+        prep_smem(k, sm);
         cudaEvent_t e = tbeg(std::is_same<U, T>::value ? 3 : 7, is_cg_epi<Epi>::value ? 3 : 0,
                              xbytes<U>(NC, rw_words<Epi>()), xflops(NC));
-        k<<<bl, th, sm * NC, st>>>(g, spec_of<U>(), epi, tw_of<U>(g.nx), partials, s);
+        k<<<x.blocks, x.threads, sm, st>>>(g, x.RP, spec_of<U>(), epi, tw_of<U>(g.nx), partials, s);
         CK(cudaGetLastError());
         tend(e);
         ++launches;
     }
     template <int NC, class Mid> void x_mid(const Mid &mid, Scal *s) { x_mid2<NC, NC>(mid, s); }
     template <int NCI, int NCO, class Mid> void x_mid2(const Mid &mid, Scal *s) {
-        int th, bl; size_t sm; xcfg(th, bl, sm);
+        const XShape x = xshape();
+        const size_t sm = x_smem<T>(g.nx, x.RP, NCI);
         auto k = k_x_mid<T, NCI, NCO, Mid>;
-        prep_smem(k, sm * NCI);
+        prep_smem(k, sm);
         cudaEvent_t e = tbeg(4, 0, xbytes(NCI + NCO, rw_words<Mid>()), xflops(NCI + NCO));
-        k<<<bl, th, sm * NCI, st>>>(g, spec, mid, tw[g.nx], s);
+        k<<<x.blocks, x.threads, sm, st>>>(g, x.RP, spec, mid, tw[g.nx], s);
         CK(cudaGetLastError());
         tend(e);
         ++launches;
@@ -1306,12 +1294,12 @@ struct Engine : EngineBase {
         const int NM = NCI > NCO ? NCI : NCO;
         int threads;
         size_t sm;
-        axis_shape<CU>(L, NM, CW, threads, sm, aw);
+        axis_shape<U>(L, NM, CW, threads, sm, aw);
         // FP64 passes of the FP32 engine: halve the tuned width until the tile fits (Px stays a
         // multiple of the narrower width)
         while (sm > 200 * 1024 && CW > 1) {
             CW >>= 1;
-            axis_shape<CU>(L, NM, CW, threads, sm, aw);
+            axis_shape<U>(L, NM, CW, threads, sm, aw);
         }
         dim3 grid(g.Px / CW, ax == 1 ? g.nz : g.ny);
         auto k = axis_kernel<U, NCI, NCO, MODE, Op>(L);
@@ -1390,26 +1378,29 @@ struct Engine : EngineBase {
     template <int NC, class Pro>
     void x_fwd_b(const std::vector<Engine *> &es, const std::vector<Pro> &fs, const std::vector<Scal *> &scs,
                  cudaStream_t s) {
-        int th, bl; size_t sm; xcfg(th, bl, sm);
+        const XShape x = xshape();
+        const size_t sm = x_smem<T>(g.nx, x.RP, NC);
         auto k = k_x_fwd_b<T, NC, Pro>;
-        prep_x(k, sm * NC);
-        k<<<dim3(bl, 1, (unsigned)es.size()), th, sm * NC, s>>>(g, slot_args(es, fs, scs), tw[g.nx]);
+        prep_x(k, sm);
+        k<<<dim3(x.blocks, 1, (unsigned)es.size()), x.threads, sm, s>>>(g, x.RP, slot_args(es, fs, scs), tw[g.nx]);
     }
     template <int NC, class Epi>
     void x_inv_b(const std::vector<Engine *> &es, const std::vector<Epi> &fs, const std::vector<Scal *> &scs,
                  cudaStream_t s) {
-        int th, bl; size_t sm; xcfg(th, bl, sm);
+        const XShape x = xshape();
+        const size_t sm = x_smem<T>(g.nx, x.RP, NC);
         auto k = k_x_inv_b<T, NC, Epi>;
-        prep_smem(k, sm * NC);
-        k<<<dim3(bl, 1, (unsigned)es.size()), th, sm * NC, s>>>(g, slot_args(es, fs, scs), tw[g.nx]);
+        prep_smem(k, sm);
+        k<<<dim3(x.blocks, 1, (unsigned)es.size()), x.threads, sm, s>>>(g, x.RP, slot_args(es, fs, scs), tw[g.nx]);
     }
     template <int NCI, int NCO, class Mid>
     void x_mid_b(const std::vector<Engine *> &es, const std::vector<Mid> &fs, const std::vector<Scal *> &scs,
                  cudaStream_t s) {
-        int th, bl; size_t sm; xcfg(th, bl, sm);
+        const XShape x = xshape();
+        const size_t sm = x_smem<T>(g.nx, x.RP, NCI);
         auto k = k_x_mid_b<T, NCI, NCO, Mid>;
-        prep_smem(k, sm * NCI);
-        k<<<dim3(bl, 1, (unsigned)es.size()), th, sm * NCI, s>>>(g, slot_args(es, fs, scs), tw[g.nx]);
+        prep_smem(k, sm);
+        k<<<dim3(x.blocks, 1, (unsigned)es.size()), x.threads, sm, s>>>(g, x.RP, slot_args(es, fs, scs), tw[g.nx]);
     }
     template <int NCI, int NCO, int MODE, class Op>
     void axis_b(int ax, const std::vector<Engine *> &es, const std::vector<Op> &fs, const std::vector<Scal *> &scs,
@@ -1419,7 +1410,7 @@ struct Engine : EngineBase {
         const int NM = NCI > NCO ? NCI : NCO;
         int threads;
         size_t sm;
-        axis_shape<C>(L, NM, CW, threads, sm, aw);
+        axis_shape<T>(L, NM, CW, threads, sm, aw);
         auto k = axis_kernel_b<T, NCI, NCO, MODE, Op>(L);
         prep_smem(k, sm);
         k<<<dim3(g.Px / CW, ax == 1 ? g.nz : g.ny, (unsigned)es.size()), threads, sm, s>>>(g, ax, CW,

@@ -3,10 +3,10 @@
 // A spectral operator  v -> F^-1[ Op(xi) F[ pro(v) ] ]  is applied as
 //   k_x_fwd   : per pair of x-rows, evaluate the prologue (e.g. the stress C_phi : p of a CG
 //               direction) for NC components, pack the two real rows as one complex line, FFT
-//               along x in shared memory, split into the two half spectra, store [c][z][y][kx];
-//   k_axis    : per tile of CW adjacent kx columns, FFT along y (2D) or y then z (3D), one warp
-//               per line in registers, apply the per-frequency operator (projection, gradient,
-//               divergence, preconditioner), inverse FFT, store;
+//               along x, split into the two half spectra, store [c][z][y][kx];
+//   k_axis    : per tile of CW adjacent kx columns, FFT along y (2D) or y then z (3D), apply the
+//               per-frequency operator (projection, gradient, divergence, preconditioner), inverse
+//               FFT, store;
 //   k_x_inv   : rebuild the packed line from two half spectra, inverse FFT along x, evaluate the
 //               epilogue (CG vector update, residual, dot products) with a deterministic
 //               reduction finalised by the last CTA.
@@ -15,9 +15,11 @@
 // so a whole CG iteration is launched without host synchronisation.
 #pragma once
 
+#include <algorithm>
 #include <type_traits>
 
 #include "pff_common.cuh"
+#include "pff_fixed.cuh"
 
 namespace pff {
 
@@ -28,283 +30,195 @@ enum { AX_FWD = 0, AX_INV = 1, AX_FWD_OP_INV = 2 };
 template <class E, class = void> struct facc_of : std::false_type {};
 template <class E> struct facc_of<E, std::void_t<decltype(E::FACC)>> : std::integral_constant<bool, E::FACC> {};
 
-// Launch bounds of the forward x pass: at most 256 threads (max(128, nx / 4)); on the FP32 path
-// at least 3 such CTAs per SM (<= 85 registers), so that more warps cover the latency of the
-// fused prologue's loads, which bound it on large grids (128^3: 174 -> 150 us per CG launch;
-// the inverse and middle x passes measured 5-10 % slower with the same bound and keep theirs).
-template <typename T> __host__ __device__ constexpr int x_max_threads() { return sizeof(T) == 4 ? 256 : 512; }
-template <typename T> __host__ __device__ constexpr int x_min_blocks() { return sizeof(T) == 4 ? 3 : 1; }
+// ---- transform of lines ----------------------------------------------------------------------------
+// FP64 lines are transformed in 64-bit fixed point (fx_lines; pff_fixed.cuh), FP32 lines in float2:
+// shared-memory Stockham (fft_lines) in the x passes, warps in registers (warp_lines) in the column passes.
+// The FP32 forms were measured against fx_lines instantiated for float2: 128^3 column pass 48 against
+// 58 us, 1024^2 column pass 25 against 42 us, x passes equal or slower.
+// `line_c` is the type that the butterflies work on, `line_w` that of the twiddles.
+template <typename T> struct line_of;
+template <> struct line_of<float> { typedef float2 c; typedef float2 w; };
+template <> struct line_of<double> { typedef fx2 c; typedef fxw w; };
+template <typename T> using line_c = typename line_of<T>::c;
+template <typename T> using line_w = typename line_of<T>::w;
 
-// ---- x-axis forward (r2c) pass ------------------------------------------------------------------
-template <typename T, int NC, class Pro>
-__device__ __forceinline__ void x_fwd_body(const Geom &g, const Pro &pro, typename cplx_of<T>::type *__restrict__ spec,
-                                           const typename cplx_of<T>::type *__restrict__ tw, double *partials,
-                                           Scal *sc) {
-    typedef typename cplx_of<T>::type C;
+__device__ __forceinline__ int ilog2(int v) { return 31 - __clz(v); }
+
+// Twiddle table of a line of L points (host side), in the form that the butterflies use.
+static inline void axis_twiddle(int m, int L, fxw &w) { w = fx_twiddle_host(m, L); }
+static inline void axis_twiddle(int m, int L, float2 &w) {
+    const long double a = -2.0L * 3.14159265358979323846264338327950288L * (long double)m / (long double)L;
+    w = make_float2((float)cosl(a), (float)sinl(a));
+}
+
+// Shared-memory index of point p of a line. FP64 lines skip one element after every eight, so that
+// the strided writes of the first exchange of fx_lines (8 t + q) hit distinct banks.
+template <typename T> __host__ __device__ __forceinline__ constexpr int lpos(int p) {
+    return sizeof(T) == 8 ? p + (p >> 3) : p;
+}
+// Elements of shared memory that an FP64 line of L points needs, a multiple of 16.
+__host__ __device__ constexpr int fx_line_room(int L) { return (L + L / 8 + 15) / 16 * 16; }
+// Stride of the lines of an x pass.
+template <typename T> __host__ __device__ constexpr int x_line_stride(int L) {
+    return sizeof(T) == 8 ? fx_line_room(L) + 4 : L;
+}
+
+
+// 4- and 8-point DFTs, natural order in and out (forward).
+__device__ __forceinline__ void fx_dft4(fx2 &a, fx2 &b, fx2 &c, fx2 &d) {
+    const fx2 p = cadd(a, c), m = csub(a, c), q = cadd(b, d), r = csub(b, d);
+    a = cadd(p, q);
+    b.x = m.x + r.y; b.y = m.y - r.x;
+    c = csub(p, q);
+    d.x = m.x - r.y; d.y = m.y + r.x;
+}
+__device__ __forceinline__ void fx_dft8(fx2 (&v)[8]) {
+    fx2 e[4], o[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        e[j] = cadd(v[j], v[j + 4]);
+        o[j] = csub(v[j], v[j + 4]);
+    }
+    // odd outputs: o_j w_8^j, w_8 = (1 - i) / sqrt 2 (the scaling before the sums: no fixed-point overflow)
+    const long long x1 = fx_mul_r2(o[1].x), y1 = fx_mul_r2(o[1].y), x3 = fx_mul_r2(o[3].x), y3 = fx_mul_r2(o[3].y);
+    o[1].x = x1 + y1; o[1].y = y1 - x1;
+    const fx2 t = o[2];
+    o[2].x = t.y; o[2].y = -t.x;
+    o[3].x = y3 - x3; o[3].y = -x3 - y3;
+    fx_dft4(e[0], e[1], e[2], e[3]);
+    fx_dft4(o[0], o[1], o[2], o[3]);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) { v[2 * j] = e[j]; v[2 * j + 1] = o[j]; }
+}
+
+// e0 of a line that holds an infinity or a NaN, or whose norm leaves the FP64 range.
+constexpr int kBadLine = 1 << 20;
+
+// Transform FP64 lines held in dynamic shared memory: line i < nlines starts at element
+// (i / NL NG + i mod NL) LS (groups of NG lines of which the first NL are transformed), point p at
+// lpos<double>(p), natural order in and out. A line of L points is worked on by T = L / 8 threads with 8
+// points each: radix-8 self-sorting passes and a last one of radix 2 or 4, each reading
+// x[t + m T] and exchanging through the line itself. 8 points per thread rather than 16: the grids
+// of this library have few lines per SM, so the work has to be spread over threads (512^2: 771 column
+// lines of 64 threads on 152 SMs). The inverse is the forward network on swapped real and
+// imaginary parts. Converts to fixed point on the way in; on the way out back to FP64 scaled by
+// 2^-osh, or leaves integers with their e0 (fx_out) in the int array at ke0 when ke0 >= 0.
+// A function of its own, called once or twice per kernel, for the build time and because one
+// instance serves every length. Every thread of the CTA calls it; blockDim is a multiple of T.
+static __device__ __noinline__ void fx_lines(int nlines, int LS, int lgL, const fxw *__restrict__ tw, bool inv, int osh,
+                                             int ke0, int NL, int NG) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C *s = reinterpret_cast<C *>(smem_raw);
-    if (pro.skip_if_done && sc->done) return;
-    const int nx = g.nx, TL = nx >> 2;
-    const int rp = threadIdx.x / TL, t = threadIdx.x - rp * TL;
-    const int RP = blockDim.x / TL;
-    const long long pair = (long long)blockIdx.x * RP + rp;
-    const int ppp = g.ny >> 1;
-    const int z = (int)(pair / ppp), y0 = 2 * (int)(pair % ppp);
-    const long long row0 = ((long long)z * g.ny + y0) * nx;
-    double acc[Pro::NR > 0 ? Pro::NR : 1];
+    __shared__ unsigned wmx[32];
+    __shared__ float wl1[32];
+    const int lgT = lgL > 3 ? lgL - 3 : 0, TH = 1 << lgT;
+    const int t = threadIdx.x & (TH - 1), gpc = blockDim.x >> lgT, nv = lgL < 3 ? 1 << lgL : 8;
+    const bool wide = TH > 32;  // a line spans several warps: CTA barriers
+    for (int first = 0; first < nlines; first += gpc) {
+        const int line = first + (threadIdx.x >> lgT);
+        const bool valid = line < nlines;
+        const int at = NL == NG ? line : line / NL * NG + line % NL;
+        double2 *p = reinterpret_cast<double2 *>(smem_raw) + (valid ? at * LS : 0);
+        fx2 *q = reinterpret_cast<fx2 *>(p);
+        double2 d[8];
+        fx2 v[8];
 #pragma unroll
-    for (int k = 0; k < (Pro::NR > 0 ? Pro::NR : 1); ++k) acc[k] = 0.0;
-    C *line = s + (size_t)rp * NC * nx;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int x = t + q * TL;
-        T va[NC], vb[NC];
-        pro.eval(row0 + x, va, acc);
-        pro.eval(row0 + nx + x, vb, acc);
-#pragma unroll
-        for (int c = 0; c < NC; ++c) line[c * nx + x] = cmk<C>(va[c], vb[c]);
-    }
-    __syncthreads();
-    fft_lines<C, NC>(s, nx, g.lx, NC, NC, 1, tw, false);
-    const int nh = (nx >> 1) + 1;
-    for (int k = t; k < nh; k += TL) {
-        const int km = (nx - k) & (nx - 1);
-#pragma unroll
-        for (int c = 0; c < NC; ++c) {
-            const C Z = line[c * nx + k], Zm = line[c * nx + km];
-            C Xa, Xb;
-            Xa.x = (T)0.5 * (Z.x + Zm.x);
-            Xa.y = (T)0.5 * (Z.y - Zm.y);
-            Xb.x = (T)0.5 * (Z.y + Zm.y);
-            Xb.y = (T)-0.5 * (Z.x - Zm.x);
-            C *dst = spec + (size_t)c * g.Nh + ((long long)z * g.ny + y0) * g.Px + k;
-            dst[0] = Xa;
-            dst[g.Px] = Xb;
+        for (int m = 0; m < 8; ++m) {
+            double2 z = make_double2(0.0, 0.0);
+            if (valid && m < nv) z = p[lpos<double>(t + (m << lgT))];
+            d[m] = inv ? make_double2(z.y, z.x) : z;
         }
-    }
-    if constexpr (Pro::NR > 0) reduce_finalize<Pro::NR>(acc, partials, sc, pro.fin(sc));
-}
-
-template <typename T, int NC, class Pro>
-__global__ void __launch_bounds__(x_max_threads<T>(), x_min_blocks<T>()) k_x_fwd(Geom g, Pro pro, typename cplx_of<T>::type *__restrict__ spec,
-                                               const typename cplx_of<T>::type *__restrict__ tw, double *partials,
-                                               Scal *sc) {
-    x_fwd_body<T, NC>(g, pro, spec, tw, partials, sc);
-}
-
-// ---- batched launches: several RVEs of one grid in one launch -----------------------------------
-// blockIdx.z selects the RVE; each carries its own functor, spectral buffer, reduction partials
-// and scalar block (the per-RVE reductions see gridDim.x * gridDim.y blocks, as unbatched).
-constexpr int kMaxBatch = 16;
-template <class F> struct SlotArg {
-    F f;
-    void *spec;
-    double *partials;
-    Scal *sc;
-};
-template <class F> struct SlotArgs {
-    SlotArg<F> a[kMaxBatch];
-};
-
-template <typename T, int NC, class Pro>
-__global__ void __launch_bounds__(x_max_threads<T>(), x_min_blocks<T>()) k_x_fwd_b(Geom g, SlotArgs<Pro> args,
-                                                 const typename cplx_of<T>::type *__restrict__ tw) {
-    typedef typename cplx_of<T>::type C;
-    const SlotArg<Pro> &a = args.a[blockIdx.z];
-    x_fwd_body<T, NC>(g, a.f, (C *)a.spec, tw, a.partials, a.sc);
-}
-
-// Load the packed complex line Z = Xa + i Xb of rows (y0, y0+1) from the half spectra.
-template <typename T, typename C>
-__device__ __forceinline__ void load_packed(const Geom &g, const C *__restrict__ spec, int c, int z, int y0,
-                                            C *line, int t, int TL) {
-    const int nx = g.nx, nh2 = nx >> 1;
-    const C *src = spec + (size_t)c * g.Nh + ((long long)z * g.ny + y0) * g.Px;
-    // TL = nx / 4, so k = t, t + TL and (for t = 0 only) t + 2 TL = nx / 2; a fixed trip count
-    // lets the loads of all three be issued together
+        // scale of the line, from its largest value and its L1 norm
+        unsigned mx = 0;
 #pragma unroll
-    for (int q = 0; q < 3; ++q) {
-        const int k = t + q * TL;
-        if (k > nh2) break;
-        C Xa = src[k], Xb = src[g.Px + k];
-        if (k == 0 || k == nh2) { Xa.y = 0; Xb.y = 0; }
-        C Z;
-        Z.x = Xa.x - Xb.y;
-        Z.y = Xa.y + Xb.x;
-        line[k] = Z;
-        if (k > 0 && k < nh2) {
-            C Zc;
-            Zc.x = Xa.x + Xb.y;
-            Zc.y = -Xa.y + Xb.x;
-            line[nx - k] = Zc;
+        for (int m = 0; m < 8; ++m) mx = max(mx, max(fx_hi_abs(d[m].x), fx_hi_abs(d[m].y)));
+        const int sw = wide ? 32 : TH;
+        for (int o = sw >> 1; o; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        const unsigned base = fx_l1_base(mx);
+        float l1 = 0.f;
+#pragma unroll
+        for (int m = 0; m < 8; ++m) l1 += fx_l1_term(fx_hi_abs(d[m].x), base) + fx_l1_term(fx_hi_abs(d[m].y), base);
+        for (int o = sw >> 1; o; o >>= 1) l1 += __shfl_xor_sync(0xffffffffu, l1, o);
+        if (wide) {
+            if ((threadIdx.x & 31) == 0) {
+                wmx[threadIdx.x >> 5] = mx;
+                wl1[threadIdx.x >> 5] = l1;
+            }
+            __syncthreads();
+            const int w0 = (threadIdx.x >> lgT) << (lgT - 5), nw = 1 << (lgT - 5);
+            for (int w = 0; w < nw; ++w) mx = max(mx, wmx[w0 + w]);
+            l1 = 0.f;
+            for (int w = 0; w < nw; ++w) {
+                const int dE = (int)(mx >> 20) - (int)(wmx[w0 + w] >> 20);
+                l1 += dE < 126 ? wl1[w0 + w] * __int_as_float((127 - dE) << 23) : 0.f;
+            }
         }
-    }
-}
-
-// ---- x-axis inverse (c2r) pass with a fused epilogue --------------------------------------------
-template <typename T, int NC, class Epi>
-__device__ __forceinline__ void x_inv_body(const Geom &g, const typename cplx_of<T>::type *__restrict__ spec,
-                                           const Epi &epi, const typename cplx_of<T>::type *__restrict__ tw,
-                                           double *partials, Scal *sc) {
-    typedef typename cplx_of<T>::type C;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    C *s = reinterpret_cast<C *>(smem_raw);
-    if (epi.skip_if_done && sc->done) return;
-    const int nx = g.nx, TL = nx >> 2;
-    const int rp = threadIdx.x / TL, t = threadIdx.x - rp * TL;
-    const int RP = blockDim.x / TL;
-    const long long pair = (long long)blockIdx.x * RP + rp;
-    const int ppp = g.ny >> 1;
-    const int z = (int)(pair / ppp), y0 = 2 * (int)(pair % ppp);
-    const long long row0 = ((long long)z * g.ny + y0) * nx;
-    C *line = s + (size_t)rp * NC * nx;
+        const int k = fx_scale(mx, l1);
+        const int e0 = mx >= 0x7ff00000u || k <= -963 ? kBadLine : 1086 - k;
 #pragma unroll
-    for (int c = 0; c < NC; ++c) load_packed<T, C>(g, spec, c, z, y0, line + c * nx, t, TL);
-    __syncthreads();
-    fft_lines<C, NC>(s, nx, g.lx, NC, NC, 1, tw, true);
-    constexpr int NR1 = Epi::NR > 0 ? Epi::NR : 1;
-    double acc[NR1];
+        for (int m = 0; m < 8; ++m) v[m] = fx2{fx_in(d[m].x, k), fx_in(d[m].y, k)};
+        for (int lgN = 0;;) {  // self-sorting passes; Ns = 2^lgN sub-transform points done
+            const int left = lgL - lgN;
+            if (left >= 3) {
+                const int kk = t & ((1 << lgN) - 1);
+                if (lgN > 0) {
 #pragma unroll
-    for (int k = 0; k < NR1; ++k) acc[k] = 0.0;
-    const T sN = (T)g.invN;
-    // FP32 path with an epilogue that supports it: the thread's 8 voxels are summed in FP32 and
-    // converted once (FP64 issues at 1/64 of the FP32 rate on this part); the reduction across
-    // threads and CTAs stays FP64
-    constexpr bool F32ACC = sizeof(T) == 4 && facc_of<Epi>::value;
-    float accf[NR1];
+                    for (int r = 1; r < 8; ++r) v[r] = cmul(v[r], tw[(r * kk) << (left - 3)]);
+                }
+                fx_dft8(v);
+                if (left == 3) break;
+                if (wide) __syncthreads();
+                else __syncwarp();
+                if (valid) {
 #pragma unroll
-    for (int k = 0; k < NR1; ++k) accf[k] = 0.f;
+                    for (int r = 0; r < 8; ++r) q[lpos<double>(((t - kk) << 3) + kk + (r << lgN))] = v[r];
+                }
+                if (wide) __syncthreads();
+                else __syncwarp();
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int x = t + q * TL;
-        T va[NC], vb[NC];
+                for (int m = 0; m < 8; ++m) v[m] = q[lpos<double>(t + (m << lgT))];
+                lgN += 3;
+            } else if (left == 2) {
+                if (lgL == 2) {
+                    fx_dft4(v[0], v[1], v[2], v[3]);
+                } else {
 #pragma unroll
-        for (int c = 0; c < NC; ++c) {
-            const C v = line[c * nx + x];
-            va[c] = v.x * sN;
-            vb[c] = v.y * sN;
+                    for (int b = 0; b < 2; ++b) {
+                        const int j = t + (b << lgT);
+#pragma unroll
+                        for (int r = 1; r < 4; ++r) v[b + 2 * r] = cmul(v[b + 2 * r], tw[r * j]);
+                        fx_dft4(v[b], v[b + 2], v[b + 4], v[b + 6]);
+                    }
+                }
+                break;
+            } else {
+#pragma unroll
+                for (int b = 0; b < 4; ++b) {
+                    const fx2 c = cmul(v[b + 4], tw[t + (b << lgT)]);
+                    v[b + 4] = csub(v[b], c);
+                    v[b] = cadd(v[b], c);
+                }
+                break;
+            }
         }
-        if constexpr (F32ACC) {
-            epi.apply_f(row0 + x, va, accf);
-            epi.apply_f(row0 + nx + x, vb, accf);
-        } else {
-            epi.apply(row0 + x, va, acc);
-            epi.apply(row0 + nx + x, vb, acc);
-        }
-    }
-    if constexpr (F32ACC) {
+        if (valid) {
+            if (ke0 >= 0) {
 #pragma unroll
-        for (int k = 0; k < NR1; ++k) acc[k] = (double)accf[k];
-    }
-    if constexpr (Epi::NR > 0) reduce_finalize<Epi::NR>(acc, partials, sc, epi.fin(sc));
-}
-
-template <typename T, int NC, class Epi>
-__global__ void __launch_bounds__(512) k_x_inv(Geom g, const typename cplx_of<T>::type *__restrict__ spec, Epi epi,
-                                               const typename cplx_of<T>::type *__restrict__ tw, double *partials,
-                                               Scal *sc) {
-    x_inv_body<T, NC>(g, spec, epi, tw, partials, sc);
-}
-
-template <typename T, int NC, class Epi>
-__global__ void __launch_bounds__(512) k_x_inv_b(Geom g, SlotArgs<Epi> args,
-                                                 const typename cplx_of<T>::type *__restrict__ tw) {
-    typedef typename cplx_of<T>::type C;
-    const SlotArg<Epi> &a = args.a[blockIdx.z];
-    x_inv_body<T, NC>(g, (const C *)a.spec, a.f, tw, a.partials, a.sc);
-}
-
-// ---- x-axis inverse, pointwise map, x-axis forward ----------------------------------------------
-// Inverse x pass of NCI components, mid.apply(v, in[NCI], out[NCO]) per voxel (NCO <= NCI), forward
-// x pass of the NCO outputs.
-template <typename T, int NCI, int NCO, class Mid>
-__device__ __forceinline__ void x_mid_body(const Geom &g, typename cplx_of<T>::type *__restrict__ spec, const Mid &mid,
-                                           const typename cplx_of<T>::type *__restrict__ tw, Scal *sc) {
-    typedef typename cplx_of<T>::type C;
-    static_assert(NCO <= NCI, "k_x_mid maps NCI components to at most NCI");
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    C *s = reinterpret_cast<C *>(smem_raw);
-    if (mid.skip_if_done && sc->done) return;
-    const int nx = g.nx, TL = nx >> 2;
-    const int rp = threadIdx.x / TL, t = threadIdx.x - rp * TL;
-    const int RP = blockDim.x / TL;
-    const long long pair = (long long)blockIdx.x * RP + rp;
-    const int ppp = g.ny >> 1;
-    const int z = (int)(pair / ppp), y0 = 2 * (int)(pair % ppp);
-    const long long row0 = ((long long)z * g.ny + y0) * nx;
-    C *line = s + (size_t)rp * NCI * nx;
+                for (int m = 0; m < 8; ++m)
+                    if (m < nv) q[lpos<double>(t + (m << lgT))] = v[m];
+                if (t == 0) (reinterpret_cast<int *>(smem_raw) + ke0)[at] = e0;
+            } else {
 #pragma unroll
-    for (int c = 0; c < NCI; ++c) load_packed<T, C>(g, spec, c, z, y0, line + c * nx, t, TL);
-    __syncthreads();
-    fft_lines<C, NCI>(s, nx, g.lx, NCI, NCI, 1, tw, true);
-    const T sN = (T)g.invN;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int x = t + q * TL;
-        T va[NCI], vb[NCI], oa[NCO], ob[NCO];
-#pragma unroll
-        for (int c = 0; c < NCI; ++c) {
-            const C v = line[c * nx + x];
-            va[c] = v.x * sN;
-            vb[c] = v.y * sN;
-        }
-        mid.apply(row0 + x, va, oa);
-        mid.apply(row0 + nx + x, vb, ob);
-#pragma unroll
-        for (int c = 0; c < NCO; ++c) line[c * nx + x] = cmk<C>(oa[c], ob[c]);
-    }
-    __syncthreads();
-    fft_lines<C, NCI>(s, nx, g.lx, NCO, NCI, 1, tw, false);
-    const int nh = (nx >> 1) + 1;
-    for (int k = t; k < nh; k += TL) {
-        const int km = (nx - k) & (nx - 1);
-#pragma unroll
-        for (int c = 0; c < NCO; ++c) {
-            const C Z = line[c * nx + k], Zm = line[c * nx + km];
-            C Xa, Xb;
-            Xa.x = (T)0.5 * (Z.x + Zm.x);
-            Xa.y = (T)0.5 * (Z.y - Zm.y);
-            Xb.x = (T)0.5 * (Z.y + Zm.y);
-            Xb.y = (T)-0.5 * (Z.x - Zm.x);
-            C *dst = spec + (size_t)c * g.Nh + ((long long)z * g.ny + y0) * g.Px + k;
-            dst[0] = Xa;
-            dst[g.Px] = Xb;
+                for (int m = 0; m < 8; ++m) {
+                    double x = fx_out(v[m].x, e0 - osh), y = fx_out(v[m].y, e0 - osh);
+                    if (e0 == kBadLine) x = y = fx_nan();
+                    if (m < nv) p[lpos<double>(t + (m << lgT))] = inv ? make_double2(y, x) : make_double2(x, y);
+                }
+            }
         }
     }
 }
 
-template <typename T, int NCI, int NCO, class Mid>
-__global__ void __launch_bounds__(512) k_x_mid(Geom g, typename cplx_of<T>::type *__restrict__ spec, Mid mid,
-                                               const typename cplx_of<T>::type *__restrict__ tw, Scal *sc) {
-    x_mid_body<T, NCI, NCO>(g, spec, mid, tw, sc);
-}
-
-template <typename T, int NCI, int NCO, class Mid>
-__global__ void __launch_bounds__(512) k_x_mid_b(Geom g, SlotArgs<Mid> args,
-                                                 const typename cplx_of<T>::type *__restrict__ tw) {
-    typedef typename cplx_of<T>::type C;
-    const SlotArg<Mid> &a = args.a[blockIdx.z];
-    x_mid_body<T, NCI, NCO>(g, (C *)a.spec, a.f, tw, a.sc);
-}
-
-
-// ---- y / z axis pass ----------------------------------------------------------------------------
-// axis = 1 (y) or 2 (z). A CTA owns CW adjacent kx columns of one plane (z for axis y, y for
-// axis z) and all L points along the axis, for every component. MODE: AX_FWD, AX_INV or
-// AX_FWD_OP_INV (forward, the per-frequency operator mapping NCI -> NCO components, inverse).
-//
-//  1. The tile is read from global memory with consecutive threads on consecutive kx (coalesced
-//     runs of CW complex values per row) into shared memory, one line of L points per
-//     (component, column). Lines are padded so that the transposing writes hit distinct banks.
-//  2. Each line is transformed by one warp (or a lane group of S = L / R lanes when L < 128) in
-//     registers: lane l holds the R points l + S m (m < R); an R-point decimation-in-frequency
-//     FFT over m, a twiddle by w_L^(l k1), then an S-point DIF across the lanes with shuffles
-//     (see wfft_fwd). No CTA barrier is taken inside a transform. The spectrum is left in the
-//     scrambled storage order of the network: position p = l + S m holds the frequency
-//     axis_freq(p) = brev_R(m) + R brev_S(l); the operator is evaluated there, and the inverse
-//     network (wfft_inv) takes that order back to natural order. In 3D the y pass stores its
-//     spectrum in storage order between the forward and the inverse y passes, so the z pass
-//     maps its plane index through axis_freq as well.
+// ---- FP32 lines of the column passes, one lane group or warp per line, in registers ------------------
 template <int R> struct log2_of { static constexpr int v = R == 1 ? 0 : 1 + log2_of<R / 2>::v; };
 template <> struct log2_of<1> { static constexpr int v = 0; };
 
@@ -319,11 +233,11 @@ __host__ __device__ constexpr bool axis_two_pass(int L) { return L >= 256; }
 __device__ __forceinline__ int brev_bits(int v, int bits) {
     return bits == 0 ? 0 : (int)(__brev((unsigned)v) >> (32 - bits));
 }
-__device__ __forceinline__ int ilog2(int v) { return 31 - __clz(v); }
 // Frequency index held at storage position p of a line of L points after the forward transform.
 // Single pass (wfft_fwd): p = l + S m holds brev_R(m) + R brev_S(l). Two-pass (wfft2_fwd, S = 32
 // lanes in G = 32 / R groups): p = l + 32 c holds brev_R(l / G) + R brev_R(c) + R^2 brev_G(l mod G).
-__device__ __forceinline__ int axis_freq(int p, int L) {
+template <typename T> __device__ __forceinline__ int axis_freq(int p, int L) {
+    if (sizeof(T) == 8) return p;  // FP64 lines are in natural order
     const int R = axis_points_per_lane(L);
     const int lgR = ilog2(R), lgS = ilog2(L) - lgR;
     if (!axis_two_pass(L)) {
@@ -336,9 +250,6 @@ __device__ __forceinline__ int axis_freq(int p, int L) {
     return brev_bits(j, lgR) + (brev_bits(c, lgR) << lgR) + (brev_bits(gg, lgG) << (2 * lgR));
 }
 
-__device__ __forceinline__ double2 shfl_xor_c(double2 v, int m) {
-    return make_double2(__shfl_xor_sync(0xffffffffu, v.x, m), __shfl_xor_sync(0xffffffffu, v.y, m));
-}
 __device__ __forceinline__ float2 shfl_xor_c(float2 v, int m) {
     return make_float2(__shfl_xor_sync(0xffffffffu, v.x, m), __shfl_xor_sync(0xffffffffu, v.y, m));
 }
@@ -347,10 +258,8 @@ template <typename C> __device__ __forceinline__ C conj_c(C a) { a.y = -a.y; ret
 // w_32^t = exp(-2 pi i t / 32), t < 32: the twiddles of the in-register stages (R <= 32), at
 // offsets known at compile time, so they are read from the constant bank. Each translation unit
 // that includes this header has its own copy; axis_twiddles_init() fills it on the current device.
-static __constant__ double2 c_w32d[32];
 static __constant__ float2 c_w32f[32];
 template <typename C> __device__ __forceinline__ C w32(int t);
-template <> __device__ __forceinline__ double2 w32<double2>(int t) { return c_w32d[t]; }
 template <> __device__ __forceinline__ float2 w32<float2>(int t) { return c_w32f[t]; }
 
 // d w_32^t and d conj(w_32^t) for a t known at compile time (the unrolled stages): t = 8 is -i,
@@ -365,16 +274,12 @@ template <typename C> __device__ __forceinline__ C mul_w32c(const C &d, int t) {
 }
 
 static inline cudaError_t axis_twiddles_init() {
-    double2 d[32];
     float2 f[32];
     for (int t = 0; t < 32; ++t) {
         const long double a = -2.0L * 3.14159265358979323846264338327950288L * (long double)t / 32.0L;
-        d[t] = make_double2((double)cosl(a), (double)sinl(a));
         f[t] = make_float2((float)cosl(a), (float)sinl(a));
     }
-    cudaError_t e = cudaMemcpyToSymbol(c_w32d, d, sizeof(d));
-    if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_w32f, f, sizeof(f));
-    return e;
+    return cudaMemcpyToSymbol(c_w32f, f, sizeof(f));
 }
 
 // Forward lane stage h over the R values of each lane: the lower lane of a pair keeps a + b, the
@@ -577,22 +482,10 @@ __device__ __forceinline__ void wfft2_inv(C (&v)[R], C *line, int l, int L, cons
     regs_dit<C, R>(v);
 }
 
-// Padding of a shared-memory line (complex elements): with CW columns read per row, the rows of
-// one 128-byte phase of a warp access land on distinct banks.
-template <typename C> __host__ __device__ constexpr int axis_line_pad(int CW) {
-    return (int)(128 / sizeof(C)) / CW;
-}
-// Stride of a shared-memory line: L plus the padding, plus room for the transposition of the
-// two-pass transform where it is used (R >= 8; 32 is a multiple of the bank period, so the
-// padding keeps its effect).
-template <typename C> __host__ __device__ constexpr int axis_line_stride(int L, int CW) {
-    return L + axis_line_pad<C>(CW) + (axis_two_pass(L) ? 32 : 0);
-}
-
 // Transform the lines [0, nlines) of the tile, one line per lane group of S lanes, looping over
 // groups of lines when there are more lines than warps. INV selects the inverse network.
 template <typename C, int R, bool TWO, bool INV>
-__device__ __forceinline__ void axis_lines(C *s, int nlines, int LS, int L, const C *__restrict__ tw) {
+__device__ __forceinline__ void warp_lines(C *s, int nlines, int LS, int L, const C *__restrict__ tw) {
     const int lgS = ilog2(L) - log2_of<R>::v, S = 1 << lgS;
     const int lpw = 32 >> lgS;  // lines per warp
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
@@ -620,9 +513,17 @@ __device__ __forceinline__ void axis_lines(C *s, int nlines, int LS, int L, cons
     }
 }
 
-// Threads per CTA at most: 512, or 256 where a lane holds 16 or more values (more registers each).
+// Stride of the lines of a column tile of CW columns. Consecutive threads read CW columns of a row, so
+// lines that differ by one start (128 bytes / CW) apart modulo the 128-byte bank period and the
+// transposing accesses of one phase hit distinct banks; FP32 lines of the two-pass form have room for
+// their transposition.
+template <typename T> __host__ __device__ constexpr int axis_line_stride(int L, int CW) {
+    return sizeof(T) == 8 ? fx_line_room(L) + 8 / CW : L + 16 / CW + (axis_two_pass(L) ? 32 : 0);
+}
+
+// Threads per CTA at most: 512, or 256 where an FP32 lane holds 16 or more values (more registers each).
 template <typename T> __host__ __device__ constexpr int axis_max_threads(int R) {
-    return (R >= 16 || (sizeof(T) == 8 && R >= 8)) ? 256 : 512;
+    return sizeof(T) == 4 && R >= 16 ? 256 : 512;
 }
 // Dispatch key of the column-pass instances: points per lane and form.
 enum { AXK_4 = 0, AXK_16 = 1, AXK_8T = 2, AXK_16T = 3, AXK_32T = 4 };
@@ -634,11 +535,345 @@ template <int K> struct axis_form_of {
     static constexpr bool TWO = K >= AXK_8T;
 };
 
+// ---- x passes ------------------------------------------------------------------------------------
+// A CTA owns RP pairs of x-rows; each pair is one packed complex line Z = a + i b per component.
+// Pointwise work runs over the RP nx columns of the pairs with every thread. Launch bounds: 256 threads,
+// 512 for the inverse and middle FP32 passes as before; on the FP32 forward path at least 3 CTAs of 256
+// threads per SM (<= 85 registers), so that more warps cover the latency of the fused prologue's loads,
+// which bound it on large grids (128^3: 174 -> 150 us per CG launch; the inverse and middle x
+// passes measured 5-10 % slower with the same bound and keep theirs).
+template <typename T> __host__ __device__ constexpr int x_max_threads() { return 256; }
+template <typename T> __host__ __device__ constexpr int x_inv_threads() { return sizeof(T) == 8 ? 256 : 512; }
+template <typename T> __host__ __device__ constexpr int x_min_blocks() { return sizeof(T) == 8 ? 2 : 3; }
+
+// Launch shape. FP32: 128 threads of 4 columns. FP64: 256 columns (256 threads from 512 columns on); on
+// small grids an FP64 pass is bound by the FP64 work of the few SMs that hold a CTA, so there a CTA
+// takes as few row pairs as give a whole warp, until there are two CTAs per SM (64^2 with the
+// split: 4 -> 32 CTAs, 66 -> 24 us per forward pass; FP32 passes gained nothing from it).
+struct XShape { int threads, blocks, RP; };
+template <typename T> inline XShape x_shape(int nx, long long pairs) {
+    constexpr bool fx = sizeof(T) == 8;
+    const int unit = fx ? nx : nx / 4;  // FP64: columns, FP32: threads of a row pair
+    const int full = fx ? 256 : 128;
+    int RP = full / unit > 1 ? full / unit : 1;
+    while (RP > 1 && (RP > pairs || (fx && pairs / RP < 304 && RP / 2 * unit >= 32))) RP >>= 1;
+    XShape x;
+    x.RP = RP;
+    x.blocks = (int)(pairs / RP);
+    x.threads = !fx ? RP * unit : (RP * nx >= 512 || x.blocks < 304 ? std::min(256, RP * nx) : std::max(32, RP * nx / 2));
+    return x;
+}
+// Dynamic shared memory: the lines, then (FP64) one exponent per line.
+template <typename T> inline size_t x_smem(int nx, int RP, int NC) {
+    return (size_t)RP * NC * (x_line_stride<T>(nx) * 2 * sizeof(T) + (sizeof(T) == 8 ? 4 : 0));
+}
+template <typename T> __device__ __forceinline__ int x_ke0(int nlines, int LS) {
+    return sizeof(T) == 8 ? nlines * LS * 4 : -1;
+}
+// Transform the first NL of the NG lines of each of the RP row pairs of the CTA.
+template <typename T, int NL, int NG>
+__device__ __forceinline__ void x_lines(typename cplx_of<T>::type *s, const Geom &g, int RP, int LS,
+                                        const line_w<T> *__restrict__ tw, bool inv, int ke0) {
+    if constexpr (sizeof(T) == 8) fx_lines(RP * NL, LS, g.lx, tw, inv, inv ? g.lx + g.ly + g.lz : 0, ke0, NL, NG);
+    else fft_lines<float2, NL>(s, g.nx, g.lx, NL, NG, 1, tw, inv);
+}
+
+// Call f(row pair, x) for the columns of the CTA's row pairs that this thread handles: FP32, four columns
+// nx / 4 apart, unrolled so that their loads are in flight together; FP64, a strided loop.
+template <typename T, class F> __device__ __forceinline__ void x_columns(const Geom &g, int RP, const F &f) {
+    if constexpr (sizeof(T) == 4) {
+        const int TL = g.nx >> 2, rp = threadIdx.x / TL, t = threadIdx.x - rp * TL;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) f(rp, t + q * TL);
+    } else {
+#pragma unroll 2
+        for (int i = threadIdx.x; i < RP * g.nx; i += blockDim.x) f(i >> g.lx, i & (g.nx - 1));
+    }
+}
+
+// Store the two half spectra of each packed line of the CTA, Xa = (Z(k) + conj Z(-k)) / 2,
+// Xb = (Z(k) - conj Z(-k)) / 2i. FP64 lines are still integers here: the sums are exact and the halving
+// goes into the exponent of the conversion.
+template <typename T, int NC, int NG>
+__device__ __forceinline__ void store_split(const Geom &g, typename cplx_of<T>::type *__restrict__ spec, long long pair0,
+                                            int RP, const typename cplx_of<T>::type *s, int LS, const int *ke) {
+    typedef typename cplx_of<T>::type C;
+    const int nx = g.nx, lh = g.lx - 1, h = 1 << lh;
+    if constexpr (sizeof(T) == 4) {
+        const int TL = nx >> 2, rp = threadIdx.x / TL, t = threadIdx.x - rp * TL;
+        for (int k = t; k <= h; k += TL) {
+            const int km = (nx - k) & (nx - 1);
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                const C *line = s + (rp * NG + c) * LS;
+                const C Z = line[k], Zm = line[km];
+                C *dst = spec + (size_t)c * g.Nh + 2 * (pair0 + rp) * g.Px + k;
+                dst[0] = make_float2(0.5f * (Z.x + Zm.x), 0.5f * (Z.y - Zm.y));
+                dst[g.Px] = make_float2(0.5f * (Z.y + Zm.y), -0.5f * (Z.x - Zm.x));
+            }
+        }
+    } else {
+        for (int i = threadIdx.x; i < RP * NC * h; i += blockDim.x) {
+            const int ln = i >> lh, k0 = i & (h - 1);
+            const int rp = ln / NC, c = ln - rp * NC, at = rp * NG + c;
+            const fx2 *line = reinterpret_cast<const fx2 *>(s + at * LS);
+            C *dst = spec + (size_t)c * g.Nh + 2 * (pair0 + rp) * g.Px;
+            const int e0 = ke[at];
+            for (int k = k0; k <= h; k += h) {  // k0 = 0 also stores the Nyquist column
+                const fx2 Z = line[lpos<T>(k)], Zm = line[lpos<T>((nx - k) & (nx - 1))];
+                C Xa = make_double2(fx_out(Z.x + Zm.x, e0 - 1), fx_out(Z.y - Zm.y, e0 - 1));
+                C Xb = make_double2(fx_out(Z.y + Zm.y, e0 - 1), fx_out(Zm.x - Z.x, e0 - 1));
+                if (e0 == kBadLine) Xa.x = Xa.y = Xb.x = Xb.y = fx_nan();
+                dst[k] = Xa;
+                dst[g.Px + k] = Xb;
+                if (k0 != 0) break;
+            }
+        }
+    }
+}
+// Load the packed lines Z = Xa + i Xb of the CTA from the half spectra, into storage order.
+template <typename T, int NC>
+__device__ __forceinline__ void load_packed(const Geom &g, const typename cplx_of<T>::type *__restrict__ spec,
+                                            long long pair0, int RP, typename cplx_of<T>::type *s, int LS) {
+    typedef typename cplx_of<T>::type C;
+    const int nx = g.nx, lh = g.lx - 1, h = 1 << lh;
+    if constexpr (sizeof(T) == 4) {
+        // k = t, t + nx / 4 and (t = 0 only) nx / 2: a fixed trip count lets the loads be issued together
+        const int TL = nx >> 2, rp = threadIdx.x / TL, t = threadIdx.x - rp * TL;
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            C *line = s + (rp * NC + c) * nx;
+            const C *src = spec + (size_t)c * g.Nh + 2 * (pair0 + rp) * g.Px;
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                const int k = t + q * TL;
+                if (k > h) break;
+                C Xa = src[k], Xb = src[g.Px + k];
+                if (k == 0 || k == h) { Xa.y = 0; Xb.y = 0; }
+                line[k] = make_float2(Xa.x - Xb.y, Xa.y + Xb.x);
+                if (k > 0 && k < h) line[nx - k] = make_float2(Xa.x + Xb.y, -Xa.y + Xb.x);
+            }
+        }
+    } else {
+#pragma unroll 4
+        for (int i = threadIdx.x; i < RP * NC * h; i += blockDim.x) {
+            const int ln = i >> lh, k = i & (h - 1);
+            const int rp = ln / NC, c = ln - rp * NC;
+            C *line = s + ln * LS;
+            const C *src = spec + (size_t)c * g.Nh + 2 * (pair0 + rp) * g.Px;
+            const C Xa = src[k], Xb = src[g.Px + k];
+            C Z = make_double2(Xa.x - Xb.y, Xa.y + Xb.x), Zc = make_double2(Xa.x + Xb.y, Xb.x - Xa.y);
+            if (k == 0) {  // the columns k = 0 and nx / 2 are real
+                Z = make_double2(Xa.x, Xb.x);
+                Zc = make_double2(src[h].x, src[g.Px + h].x);
+            }
+            line[lpos<T>(k)] = Z;
+            line[lpos<T>(k == 0 ? h : nx - k)] = Zc;
+        }
+    }
+}
+
+// ---- x-axis forward (r2c) pass ------------------------------------------------------------------
+template <typename T, int NC, class Pro>
+__device__ __forceinline__ void x_fwd_body(const Geom &g, int RP, const Pro &pro,
+                                           typename cplx_of<T>::type *__restrict__ spec,
+                                           const line_w<T> *__restrict__ tw, double *partials, Scal *sc) {
+    typedef typename cplx_of<T>::type C;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    C *s = reinterpret_cast<C *>(smem_raw);
+    if (pro.skip_if_done && sc->done) return;
+    const int nx = g.nx, LS = x_line_stride<T>(nx);
+    const long long pair0 = (long long)blockIdx.x * RP;
+    double acc[Pro::NR > 0 ? Pro::NR : 1];
+#pragma unroll
+    for (int k = 0; k < (Pro::NR > 0 ? Pro::NR : 1); ++k) acc[k] = 0.0;
+    x_columns<T>(g, RP, [&](int rp, int x) {
+        const long long v = 2 * (pair0 + rp) * nx + x;
+        T va[NC], vb[NC];
+        pro.eval(v, va, acc);
+        pro.eval(v + nx, vb, acc);
+        C *line = s + rp * NC * LS + lpos<T>(x);
+#pragma unroll
+        for (int c = 0; c < NC; ++c) line[c * LS] = cmk<C>(va[c], vb[c]);
+    });
+    __syncthreads();
+    const int ke0 = x_ke0<T>(RP * NC, LS);
+    x_lines<T, NC, NC>(s, g, RP, LS, tw, false, ke0);
+    __syncthreads();
+    store_split<T, NC, NC>(g, spec, pair0, RP, s, LS, reinterpret_cast<int *>(smem_raw) + ke0);
+    if constexpr (Pro::NR > 0) reduce_finalize<Pro::NR>(acc, partials, sc, pro.fin(sc));
+}
+
+template <typename T, int NC, class Pro>
+__global__ void __launch_bounds__(x_max_threads<T>(), x_min_blocks<T>())
+    k_x_fwd(Geom g, int RP, Pro pro, typename cplx_of<T>::type *__restrict__ spec, const line_w<T> *__restrict__ tw,
+            double *partials, Scal *sc) {
+    x_fwd_body<T, NC>(g, RP, pro, spec, tw, partials, sc);
+}
+
+// ---- batched launches: several RVEs of one grid in one launch -----------------------------------
+// blockIdx.z selects the RVE; each carries its own functor, spectral buffer, reduction partials
+// and scalar block (the per-RVE reductions see gridDim.x * gridDim.y blocks, as unbatched).
+constexpr int kMaxBatch = 16;
+template <class F> struct SlotArg {
+    F f;
+    void *spec;
+    double *partials;
+    Scal *sc;
+};
+template <class F> struct SlotArgs {
+    SlotArg<F> a[kMaxBatch];
+};
+
+template <typename T, int NC, class Pro>
+__global__ void __launch_bounds__(x_max_threads<T>(), x_min_blocks<T>())
+    k_x_fwd_b(Geom g, int RP, SlotArgs<Pro> args, const line_w<T> *__restrict__ tw) {
+    typedef typename cplx_of<T>::type C;
+    const SlotArg<Pro> &a = args.a[blockIdx.z];
+    x_fwd_body<T, NC>(g, RP, a.f, (C *)a.spec, tw, a.partials, a.sc);
+}
+
+// ---- x-axis inverse (c2r) pass with a fused epilogue --------------------------------------------
+template <typename T, int NC, class Epi>
+__device__ __forceinline__ void x_inv_body(const Geom &g, int RP, const typename cplx_of<T>::type *__restrict__ spec,
+                                           const Epi &epi, const line_w<T> *__restrict__ tw, double *partials,
+                                           Scal *sc) {
+    typedef typename cplx_of<T>::type C;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    C *s = reinterpret_cast<C *>(smem_raw);
+    if (epi.skip_if_done && sc->done) return;
+    const int nx = g.nx, LS = x_line_stride<T>(nx);
+    const long long pair0 = (long long)blockIdx.x * RP;
+    load_packed<T, NC>(g, spec, pair0, RP, s, LS);
+    __syncthreads();
+    // the scale 1/N is a power of two: in the exponent of the FP64 conversion, a factor in FP32
+    x_lines<T, NC, NC>(s, g, RP, LS, tw, true, -1);
+    __syncthreads();
+    constexpr int NR1 = Epi::NR > 0 ? Epi::NR : 1;
+    double acc[NR1];
+#pragma unroll
+    for (int k = 0; k < NR1; ++k) acc[k] = 0.0;
+    const T sN = sizeof(T) == 8 ? (T)1 : (T)g.invN;
+    // FP32 path with an epilogue that supports it: the thread's voxels are summed in FP32 and
+    // converted once (FP64 issues at 1/64 of the FP32 rate on this part); the reduction across
+    // threads and CTAs stays FP64
+    constexpr bool F32ACC = sizeof(T) == 4 && facc_of<Epi>::value;
+    float accf[NR1];
+#pragma unroll
+    for (int k = 0; k < NR1; ++k) accf[k] = 0.f;
+    x_columns<T>(g, RP, [&](int rp, int x) {
+        const long long v = 2 * (pair0 + rp) * nx + x;
+        const C *line = s + rp * NC * LS + lpos<T>(x);
+        T va[NC], vb[NC];
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            const C z = line[c * LS];
+            va[c] = sizeof(T) == 8 ? z.x : z.x * sN;
+            vb[c] = sizeof(T) == 8 ? z.y : z.y * sN;
+        }
+        if constexpr (F32ACC) {
+            epi.apply_f(v, va, accf);
+            epi.apply_f(v + nx, vb, accf);
+        } else {
+            epi.apply(v, va, acc);
+            epi.apply(v + nx, vb, acc);
+        }
+    });
+    if constexpr (F32ACC) {
+#pragma unroll
+        for (int k = 0; k < NR1; ++k) acc[k] = (double)accf[k];
+    }
+    if constexpr (Epi::NR > 0) reduce_finalize<Epi::NR>(acc, partials, sc, epi.fin(sc));
+}
+
+template <typename T, int NC, class Epi>
+__global__ void __launch_bounds__(x_inv_threads<T>(), sizeof(T) == 8 ? 2 : 1)
+    k_x_inv(Geom g, int RP, const typename cplx_of<T>::type *__restrict__ spec, Epi epi,
+            const line_w<T> *__restrict__ tw, double *partials, Scal *sc) {
+    x_inv_body<T, NC>(g, RP, spec, epi, tw, partials, sc);
+}
+
+template <typename T, int NC, class Epi>
+__global__ void __launch_bounds__(x_inv_threads<T>(), sizeof(T) == 8 ? 2 : 1)
+    k_x_inv_b(Geom g, int RP, SlotArgs<Epi> args, const line_w<T> *__restrict__ tw) {
+    typedef typename cplx_of<T>::type C;
+    const SlotArg<Epi> &a = args.a[blockIdx.z];
+    x_inv_body<T, NC>(g, RP, (const C *)a.spec, a.f, tw, a.partials, a.sc);
+}
+
+// ---- x-axis inverse, pointwise map, x-axis forward ----------------------------------------------
+// Inverse x pass of NCI components, mid.apply(v, in[NCI], out[NCO]) per voxel (NCO <= NCI), forward
+// x pass of the NCO outputs.
+template <typename T, int NCI, int NCO, class Mid>
+__device__ __forceinline__ void x_mid_body(const Geom &g, int RP, typename cplx_of<T>::type *__restrict__ spec,
+                                           const Mid &mid, const line_w<T> *__restrict__ tw, Scal *sc) {
+    typedef typename cplx_of<T>::type C;
+    static_assert(NCO <= NCI, "k_x_mid maps NCI components to at most NCI");
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    C *s = reinterpret_cast<C *>(smem_raw);
+    if (mid.skip_if_done && sc->done) return;
+    const int nx = g.nx, LS = x_line_stride<T>(nx);
+    const long long pair0 = (long long)blockIdx.x * RP;
+    load_packed<T, NCI>(g, spec, pair0, RP, s, LS);
+    __syncthreads();
+    x_lines<T, NCI, NCI>(s, g, RP, LS, tw, true, -1);
+    __syncthreads();
+    const T sN = sizeof(T) == 8 ? (T)1 : (T)g.invN;
+    x_columns<T>(g, RP, [&](int rp, int x) {
+        const long long v = 2 * (pair0 + rp) * nx + x;
+        C *line = s + rp * NCI * LS + lpos<T>(x);
+        T va[NCI], vb[NCI], oa[NCO], ob[NCO];
+#pragma unroll
+        for (int c = 0; c < NCI; ++c) {
+            const C z = line[c * LS];
+            va[c] = sizeof(T) == 8 ? z.x : z.x * sN;
+            vb[c] = sizeof(T) == 8 ? z.y : z.y * sN;
+        }
+        mid.apply(v, va, oa);
+        mid.apply(v + nx, vb, ob);
+#pragma unroll
+        for (int c = 0; c < NCO; ++c) line[c * LS] = cmk<C>(oa[c], ob[c]);
+    });
+    __syncthreads();
+    const int ke0 = x_ke0<T>(RP * NCI, LS);
+    x_lines<T, NCO, NCI>(s, g, RP, LS, tw, false, ke0);
+    __syncthreads();
+    store_split<T, NCO, NCI>(g, spec, pair0, RP, s, LS, reinterpret_cast<int *>(smem_raw) + ke0);
+}
+
+template <typename T, int NCI, int NCO, class Mid>
+__global__ void __launch_bounds__(x_inv_threads<T>(), sizeof(T) == 8 ? 2 : 1)
+    k_x_mid(Geom g, int RP, typename cplx_of<T>::type *__restrict__ spec, Mid mid, const line_w<T> *__restrict__ tw,
+            Scal *sc) {
+    x_mid_body<T, NCI, NCO>(g, RP, spec, mid, tw, sc);
+}
+
+template <typename T, int NCI, int NCO, class Mid>
+__global__ void __launch_bounds__(x_inv_threads<T>(), sizeof(T) == 8 ? 2 : 1)
+    k_x_mid_b(Geom g, int RP, SlotArgs<Mid> args, const line_w<T> *__restrict__ tw) {
+    typedef typename cplx_of<T>::type C;
+    const SlotArg<Mid> &a = args.a[blockIdx.z];
+    x_mid_body<T, NCI, NCO>(g, RP, (C *)a.spec, a.f, tw, a.sc);
+}
+
+// ---- y / z axis pass ----------------------------------------------------------------------------
+// axis = 1 (y) or 2 (z). A CTA owns CW adjacent kx columns of one plane (z for axis y, y for
+// axis z) and all L points along the axis, for every component. MODE: AX_FWD, AX_INV or
+// AX_FWD_OP_INV (forward, the per-frequency operator mapping NCI -> NCO components, inverse).
+// The tile is read from global memory with consecutive threads on consecutive kx (coalesced runs
+// of CW complex values per row) into shared memory, one line of L points per (component, column).
+template <typename T, int K, bool INV>
+__device__ __forceinline__ void axis_lines(typename cplx_of<T>::type *s, int nlines, int LS, int lgL,
+                                           const line_w<T> *__restrict__ tw) {
+    if constexpr (sizeof(T) == 8) fx_lines(nlines, LS, lgL, tw, INV, 0, -1, 1, 1);
+    else warp_lines<float2, axis_form_of<K>::R, axis_form_of<K>::TWO, INV>(s, nlines, LS, 1 << lgL, tw);
+}
+
 template <typename T, int NCI, int NCO, int MODE, int K, class Op>
 __device__ __forceinline__ void axis_body(const Geom &g, int axis, int CW,
                                           const typename cplx_of<T>::type *__restrict__ spec_in,
                                           typename cplx_of<T>::type *spec_out, const Op &op,
-                                          const typename cplx_of<T>::type *__restrict__ tw, Scal *sc) {
+                                          const line_w<T> *__restrict__ tw, Scal *sc) {
     typedef typename cplx_of<T>::type C;
     constexpr int NOUT = (MODE == AX_FWD_OP_INV) ? NCO : NCI;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -647,7 +882,7 @@ __device__ __forceinline__ void axis_body(const Geom &g, int axis, int CW,
     const int L = axis == 1 ? g.ny : g.nz;
     const int lgL = axis == 1 ? g.ly : g.lz;
     const int lgCW = ilog2(CW);
-    const int LS = axis_line_stride<C>(L, CW);
+    const int LS = axis_line_stride<T>(L, CW);
     const int kx0 = blockIdx.x * CW;
     const int other = blockIdx.y;
     // element offsets in 32 bits: every spectrum of a valid configuration (at most 2^24 voxels,
@@ -681,32 +916,30 @@ __device__ __forceinline__ void axis_body(const Geom &g, int axis, int CW,
                 const int c = i >> (lgL + lgCW);
                 const int rem = i & (npt - 1);
                 const int pos = rem >> lgCW, cc = rem & (CW - 1);
-                s[((c << lgCW) + cc) * LS + pos] = tmp[u];
+                s[((c << lgCW) + cc) * LS + lpos<T>(pos)] = tmp[u];
             }
         }
     }
     __syncthreads();
     // 2. transforms (and the operator between them)
-    constexpr int R = axis_form_of<K>::R;
-    constexpr bool TWO = axis_form_of<K>::TWO;
-    axis_lines<C, R, TWO, MODE == AX_INV>(s, NCI * CW, LS, L, tw);
+    axis_lines<T, K, MODE == AX_INV>(s, NCI * CW, LS, lgL, tw);
     if constexpr (MODE == AX_FWD_OP_INV) {
         __syncthreads();
         for (int i = threadIdx.x; i < npt; i += nth) {
             const int cc = i >> lgL, p = i & (L - 1);
-            const int kk = axis_freq(p, L);
+            const int kk = axis_freq<T>(p, L);
             const int kx = kx0 + cc;
-            const int ky = axis == 1 ? kk : axis_freq(other, g.ny);
+            const int ky = axis == 1 ? kk : axis_freq<T>(other, g.ny);
             const int kz = axis == 1 ? (g.nz > 1 ? other : 0) : kk;
             C in[NCI], out[NCO];
 #pragma unroll
-            for (int c = 0; c < NCI; ++c) in[c] = s[((c << lgCW) + cc) * LS + p];
+            for (int c = 0; c < NCI; ++c) in[c] = s[((c << lgCW) + cc) * LS + lpos<T>(p)];
             op.apply(g, kx, ky, kz, in, out);
 #pragma unroll
-            for (int c = 0; c < NCO; ++c) s[((c << lgCW) + cc) * LS + p] = out[c];
+            for (int c = 0; c < NCO; ++c) s[((c << lgCW) + cc) * LS + lpos<T>(p)] = out[c];
         }
         __syncthreads();
-        axis_lines<C, R, TWO, true>(s, NCO * CW, LS, L, tw);
+        axis_lines<T, K, true>(s, NCO * CW, LS, lgL, tw);
     }
     __syncthreads();
     // 3. coalesced store
@@ -714,48 +947,47 @@ __device__ __forceinline__ void axis_body(const Geom &g, int axis, int CW,
         const int c = i >> (lgL + lgCW);
         const int rem = i & (npt - 1);
         const int pos = rem >> lgCW, cc = rem & (CW - 1);
-        spec_out[c * Nh + base + pos * lstride + cc] = s[((c << lgCW) + cc) * LS + pos];
+        spec_out[c * Nh + base + pos * lstride + cc] = s[((c << lgCW) + cc) * LS + lpos<T>(pos)];
     }
 }
 
 template <typename T, int NCI, int NCO, int MODE, int K, class Op>
 __global__ void __launch_bounds__(axis_max_threads<T>(axis_form_of<K>::R))
     k_axis(Geom g, int axis, int CW, const typename cplx_of<T>::type *__restrict__ spec_in,
-           typename cplx_of<T>::type *spec_out, Op op, const typename cplx_of<T>::type *__restrict__ tw, Scal *sc) {
+           typename cplx_of<T>::type *spec_out, Op op, const line_w<T> *__restrict__ tw, Scal *sc) {
     axis_body<T, NCI, NCO, MODE, K>(g, axis, CW, spec_in, spec_out, op, tw, sc);
 }
 
 template <typename T, int NCI, int NCO, int MODE, int K, class Op>
 __global__ void __launch_bounds__(axis_max_threads<T>(axis_form_of<K>::R))
-    k_axis_b(Geom g, int axis, int CW, SlotArgs<Op> args, const typename cplx_of<T>::type *__restrict__ tw) {
+    k_axis_b(Geom g, int axis, int CW, SlotArgs<Op> args, const line_w<T> *__restrict__ tw) {
     typedef typename cplx_of<T>::type C;
     const SlotArg<Op> &a = args.a[blockIdx.z];
     axis_body<T, NCI, NCO, MODE, K>(g, axis, CW, (const C *)a.spec, (C *)a.spec, a.f, tw, a.sc);
 }
 
-
-// Launch shape of k_axis for an axis of L points, NM components and CW columns per CTA: one lane
-// group of S = L / R lanes per line, at most 16 warps (the warps loop over the lines beyond), and
-// the padded lines in dynamic shared memory.
-template <typename C> inline void axis_shape(int L, int NM, int CW, int &threads, size_t &smem, int wcap = 16) {
-    const int R = axis_points_per_lane(L), S = L / R;
+// Launch shape of k_axis for an axis of L points, NM components and CW columns per CTA: the threads of
+// every line (FP64: L / 8 per line, FP32: a lane group of S = L / R) up to 16 warps, which loop over the
+// lines beyond, and the padded lines in dynamic shared memory.
+template <typename T> inline void axis_shape(int L, int NM, int CW, int &threads, size_t &smem, int wcap = 16) {
+    constexpr bool fx = sizeof(T) == 8;
+    const int R = fx ? 8 : axis_points_per_lane(L), S = L > R ? L / R : 1;
     const long long lanes = (long long)NM * CW * S;
-    long long w = (lanes + 31) / 32;
-    int wmax = axis_max_threads<typename real_of<C>::type>(R) / 32;
-    if (wcap >= 1 && wcap < wmax) wmax = wcap;
-    if (w > wmax) w = wmax;
-    if (w < 1) w = 1;
-    threads = (int)(32 * w);
-    smem = (size_t)NM * CW * (size_t)axis_line_stride<C>(L, CW) * sizeof(C);
+    int w = (int)std::min<long long>((lanes + 31) / 32, axis_max_threads<T>(R) / 32);
+    w = std::max(1, std::min(w, std::max(1, wcap)));
+    if (fx && S > 32) w = std::max(1, w / (S / 32)) * (S / 32);  // whole lines
+    threads = 32 * w;
+    smem = (size_t)NM * CW * (size_t)axis_line_stride<T>(L, CW) * 2 * sizeof(T);
 }
 
 template <typename T, class Op>
 using axis_kernel_t = void (*)(Geom, int, int, const typename cplx_of<T>::type *__restrict__, typename cplx_of<T>::type *,
-                               Op, const typename cplx_of<T>::type *__restrict__, Scal *);
+                               Op, const line_w<T> *__restrict__, Scal *);
 
 // The instance of k_axis for the points per lane of an axis of L points.
 template <typename T, int NCI, int NCO, int MODE, class Op> inline axis_kernel_t<T, Op> axis_kernel(int L) {
-    switch (axis_form(L)) {
+    if constexpr (sizeof(T) == 8) return k_axis<T, NCI, NCO, MODE, AXK_4, Op>;  // one instance for every length
+    else switch (axis_form(L)) {
     case AXK_4: return k_axis<T, NCI, NCO, MODE, AXK_4, Op>;
     case AXK_16: return k_axis<T, NCI, NCO, MODE, AXK_16, Op>;
     case AXK_8T: return k_axis<T, NCI, NCO, MODE, AXK_8T, Op>;
@@ -765,9 +997,10 @@ template <typename T, int NCI, int NCO, int MODE, class Op> inline axis_kernel_t
 }
 
 template <typename T, class Op>
-using axis_kernel_b_t = void (*)(Geom, int, int, SlotArgs<Op>, const typename cplx_of<T>::type *__restrict__);
+using axis_kernel_b_t = void (*)(Geom, int, int, SlotArgs<Op>, const line_w<T> *__restrict__);
 template <typename T, int NCI, int NCO, int MODE, class Op> inline axis_kernel_b_t<T, Op> axis_kernel_b(int L) {
-    switch (axis_form(L)) {
+    if constexpr (sizeof(T) == 8) return k_axis_b<T, NCI, NCO, MODE, AXK_4, Op>;  // one instance for every length
+    else switch (axis_form(L)) {
     case AXK_4: return k_axis_b<T, NCI, NCO, MODE, AXK_4, Op>;
     case AXK_16: return k_axis_b<T, NCI, NCO, MODE, AXK_16, Op>;
     case AXK_8T: return k_axis_b<T, NCI, NCO, MODE, AXK_8T, Op>;

@@ -63,12 +63,21 @@ __global__ void k_xi(double *xi, int n, int len, int half) {
     xi[k] = v;
 }
 
-__global__ void k_twiddles(double2 *tw, int L) {
+// Twiddles in the fixed-point form of the FP64 transforms.
+__global__ void k_twiddles(fxw *tw, int L) {
     int m = blockIdx.x * blockDim.x + threadIdx.x;
     if (m >= L) return;
     double s, c;
     sincospi(-2.0 * (double)m / (double)L, &s, &c);
-    tw[m] = make_double2(c, s);
+    auto put = [](double v, int &h, int &l) {
+        v *= 1073741824.0;
+        h = (int)rint(v);
+        l = (int)rint((v - (double)h) * 2147483648.0);
+    };
+    fxw w;
+    put(c, w.rh, w.rl);
+    put(s, w.ih, w.il);
+    tw[m] = w;
 }
 
 // Epilogue of the last pass: the dissipation density of Eq. (CrackLenght_ani) summed with and
@@ -138,21 +147,18 @@ extern "C" int rve_dissipation_noalloc(int dim, const int n[3], double ell, int 
     g.Nh = (long long)g.Px * ny * nz;
     g.invN = 1.0 / (double)g.N;
 
-    // launch shape of the x passes (same rule as the engine)
+    // launch shape of the x passes (same rule as the engine); grids too small for one warp of row
+    // pairs of nx / 4 columns are refused, as by rve_create
     const int TL = nx / 4;
     const long long pairs = (long long)ny * nz / 2;
-    int RP = 128 / TL;
-    if (RP < 1) RP = 1;
-    if (RP > pairs) RP = (int)pairs;
-    const int xthreads = RP * TL;
-    const int xblocks = (int)(pairs / RP);
-    if (xthreads < 32) return RVE_EINVAL;  // the x passes reduce with full-warp shuffles
+    if ((long long)TL * (128 / TL < 1 ? 1 : (128 / TL < pairs ? 128 / TL : pairs)) < 32) return RVE_EINVAL;
+    const XShape xs = x_shape<double>(nx, pairs);
 
     // scratch layout; reject grids whose requirement exceeds the static array
     Layout lay;
     lay.scal = 0;
     lay.partials = align256(sizeof(Scal));
-    lay.tw = lay.partials + align256(sizeof(double) * 2 * (size_t)xblocks);
+    lay.tw = lay.partials + align256(sizeof(double) * 2 * (size_t)xs.blocks);
     lay.xi = lay.tw + align256(sizeof(double2) * (size_t)(nx + ny + nz));
     lay.spec = lay.xi + align256(sizeof(double) * (size_t)(g.Px + ny + nz));
     lay.total = lay.spec + align256(sizeof(double2) * (size_t)dim * (size_t)g.Nh);
@@ -170,16 +176,14 @@ extern "C" int rve_dissipation_noalloc(int dim, const int n[3], double ell, int 
         // g_scratch is not a device address, so look the address up and keep it.
         void *p = nullptr;
         if (cudaGetSymbolAddress(&p, g_scratch) != cudaSuccess || !p) return RVE_ECUDA;
-        // the column passes read their in-register twiddles from this file's constant bank
-        if (axis_twiddles_init() != cudaSuccess) return RVE_ECUDA;
         g_scratch_addr[dev] = p;
     }
     unsigned char *base = (unsigned char *)g_scratch_addr[dev];
     Scal *sc = (Scal *)(base + lay.scal);
     double *partials = (double *)(base + lay.partials);
-    double2 *twx = (double2 *)(base + lay.tw);
-    double2 *twy = twx + nx;
-    double2 *twz = twy + ny;
+    fxw *twx = (fxw *)(base + lay.tw);
+    fxw *twy = twx + nx;
+    fxw *twz = twy + ny;
     double *xix = (double *)(base + lay.xi);
     double *xiy = xix + g.Px;
     double *xiz = xiy + ny;
@@ -198,13 +202,12 @@ extern "C" int rve_dissipation_noalloc(int dim, const int n[3], double ell, int 
     k_xi<<<(ny + 255) / 256, 256, 0, st>>>(xiy, ny, ny, 0);
     k_xi<<<(nz + 255) / 256, 256, 0, st>>>(xiz, nz, nz, 0);
 
-    const size_t smx = (size_t)RP * nx * sizeof(double2);
-    auto axis_launch = [&](auto kernel, int ax, int NM, const auto &op, const double2 *tw) -> cudaError_t {
+    auto axis_launch = [&](auto kernel, int ax, int NM, const auto &op, const fxw *tw) -> cudaError_t {
         const int L = ax == 1 ? ny : nz;
         const int CW = ax == 1 ? cwy : cwz;
         int threads;
         size_t sm;
-        axis_shape<double2>(L, NM, CW, threads, sm);
+        axis_shape<double>(L, NM, CW, threads, sm);
         if (sm > 32 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         kernel<<<dim3(g.Px / CW, ax == 1 ? nz : ny), threads, sm, st>>>(g, ax, CW, spec, spec, op, tw, sc);
         return cudaGetLastError();
@@ -213,7 +216,9 @@ extern "C" int rve_dissipation_noalloc(int dim, const int n[3], double ell, int 
     // forward x pass of phi
     {
         auto k = k_x_fwd<double, 1, ProField<double>>;
-        k<<<xblocks, xthreads, smx, st>>>(g, ProField<double>{false, phi}, spec, twx, partials, sc);
+        const size_t sm = x_smem<double>(nx, xs.RP, 1);
+        if (sm > 32 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        k<<<xs.blocks, xs.threads, sm, st>>>(g, xs.RP, ProField<double>{false, phi}, spec, twx, partials, sc);
         if (cudaGetLastError() != cudaSuccess) return RVE_ECUDA;
     }
     const int32_t *gid = grain_id;
@@ -221,9 +226,9 @@ extern "C" int rve_dissipation_noalloc(int dim, const int n[3], double ell, int 
         if (axis_launch(axis_kernel<double, 1, 2, AX_FWD_OP_INV, OpGrad<double2, 2>>(ny), 1, 2, OpGrad<double2, 2>{false, xi}, twy))
             return RVE_ECUDA;
         auto k = k_x_inv<double, 2, EpiDissChecked<2>>;
-        const size_t sm = smx * 2;
+        const size_t sm = x_smem<double>(nx, xs.RP, 2);
         if (sm > 32 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        k<<<xblocks, xthreads, sm, st>>>(g, spec, EpiDissChecked<2>{false, phi, Gc, A, gid, n_grains, ell}, twx,
+        k<<<xs.blocks, xs.threads, sm, st>>>(g, xs.RP, spec, EpiDissChecked<2>{false, phi, Gc, A, gid, n_grains, ell}, twx,
                                          partials, sc);
     } else {
         if (nz == 1) {
@@ -241,9 +246,9 @@ extern "C" int rve_dissipation_noalloc(int dim, const int n[3], double ell, int 
                 return RVE_ECUDA;
         }
         auto k = k_x_inv<double, 3, EpiDissChecked<3>>;
-        const size_t sm = smx * 3;
+        const size_t sm = x_smem<double>(nx, xs.RP, 3);
         if (sm > 32 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        k<<<xblocks, xthreads, sm, st>>>(g, spec, EpiDissChecked<3>{false, phi, Gc, A, gid, n_grains, ell}, twx,
+        k<<<xs.blocks, xs.threads, sm, st>>>(g, xs.RP, spec, EpiDissChecked<3>{false, phi, Gc, A, gid, n_grains, ell}, twx,
                                          partials, sc);
     }
     if (cudaGetLastError() != cudaSuccess) return RVE_ECUDA;
