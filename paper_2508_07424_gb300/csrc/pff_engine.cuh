@@ -156,13 +156,6 @@ static __global__ void k_crack_setup(long long N, int nx, int ny, const int *gid
     phi_disc[v] = pd;
 }
 
-// Loop condition of a solve captured as a conditional (while) graph node: keep iterating while
-// the device scalars say the solve is not done. The solve always ends: the update kernels set
-// done at convergence, at the iteration cap, on breakdown and on a non-finite scalar.
-static __global__ void k_loop_cond(cudaGraphConditionalHandle h, const Scal *sc) {
-    cudaGraphSetConditional(h, sc->done ? 0u : 1u);
-}
-
 static __global__ void k_init_scal(Scal *sc, double tol2, int max_iters, double abar, double bbar, double eta2) {
     sc->done = 0; sc->flag = 0; sc->iters = 0; sc->first = 1; sc->max_iters = max_iters;
     sc->tol2 = tol2; sc->beta = 0.0; sc->alpha = 0.0; sc->counter = 0u; sc->abar = abar; sc->bbar = bbar;
@@ -825,13 +818,18 @@ struct Engine : EngineBase {
     std::map<std::tuple<int, const void *, const void *>, GraphEntry> graphs;
     bool use_graphs = true;
 
-    // Whole iterative solves as one graph launch: a conditional while node whose body is one
-    // iteration plus k_loop_cond. Built once per key by capturing `body` into the node's body
-    // graph; returns false (caller falls back to chunks) when graphs are off or timing is on.
+    // Whole iterative solves as one graph launch: a conditional while node whose body is kLoopUnroll
+    // iterations. The last kernel of an iteration sets the loop condition from the device scalars
+    // (loop_cond, with the handle in cap_cond while the body is captured); the solve always ends: the
+    // update kernels set done at convergence, at the iteration cap, on breakdown and on a non-finite
+    // scalar, and later iterations of the body skip. Built once per key by capturing `body` into the
+    // node's body graph; returns false (caller falls back to chunks) when graphs are off or timing is on.
+    static constexpr int kLoopUnroll = 2;
+    cudaGraphConditionalHandle cap_cond = 0;
     struct LoopEntry { cudaGraphExec_t exec; long body_nodes; bool failed; };
     std::map<std::tuple<int, const void *, const void *>, LoopEntry> loops;
     bool use_loops = true;
-    template <class F> bool run_loop(int kind, const void *a, const void *b, Scal *s, F &&body) {
+    template <class F> bool run_loop(int kind, const void *a, const void *b, F &&body) {
         if (!use_graphs || !use_loops || timing) return false;
         auto key = std::make_tuple(kind, a, b);
         auto it = loops.find(key);
@@ -860,12 +858,12 @@ struct Engine : EngineBase {
                                                    cudaStreamCaptureModeThreadLocal) == cudaSuccess;
                 if (ok) {
                     try {
-                        body();
-                        k_loop_cond<<<1, 1, 0, st>>>(h, s);
-                        ++launches;
+                        cap_cond = h;
+                        for (int u = 0; u < kLoopUnroll; ++u) body();
                     } catch (...) {
                         ok = false;
                     }
+                    cap_cond = 0;
                     cudaGraph_t out_g;
                     ok = (cudaStreamEndCapture(cap_st, &out_g) == cudaSuccess) && ok;
                 }
@@ -886,7 +884,7 @@ struct Engine : EngineBase {
     }
     void count_loop(int kind, const void *a, const void *b, int iters) {
         auto it = loops.find(std::make_tuple(kind, a, b));
-        if (it != loops.end() && !it->second.failed) launches += (long)std::max(1, iters) * it->second.body_nodes;
+        if (it != loops.end() && !it->second.failed) launches += (long)((std::max(1, iters) + kLoopUnroll - 1) / kLoopUnroll) * it->second.body_nodes;
     }
 
     // Run `body` (which launches one chunk on `st`) as a replay of a cached CUDA graph; the first
@@ -1262,14 +1260,14 @@ struct Engine : EngineBase {
         tend(e);
         ++launches;
     }
-    template <int NC, class Epi, typename U = T> void x_inv(const Epi &epi, Scal *s) {
+    template <int NC, class Epi, typename U = T> void x_inv(const Epi &epi, Scal *s, cudaGraphConditionalHandle cond = 0) {
         const XShape x = xshape<U>();
         const size_t sm = x_smem<U>(g.nx, x.RP, NC);
         auto k = k_x_inv<U, NC, Epi>;
         prep_smem(k, sm);
         cudaEvent_t e = tbeg(std::is_same<U, T>::value ? 3 : 7, is_cg_epi<Epi>::value ? 3 : 0,
                              xbytes<U>(NC, rw_words<Epi>()), xflops(NC));
-        k<<<x.blocks, x.threads, sm, st>>>(g, x.RP, spec_of<U>(), epi, tw_of<U>(g.nx), partials, s);
+        k<<<x.blocks, x.threads, sm, st>>>(g, x.RP, spec_of<U>(), epi, tw_of<U>(g.nx), partials, s, cond);
         CK(cudaGetLastError());
         tend(e);
         ++launches;
@@ -1333,9 +1331,9 @@ struct Engine : EngineBase {
         const long long cap = F::NR > 0 ? 2LL * num_sms : 1184;
         return bl > cap ? cap : bl;
     }
-    template <class F> void pointwise(const F &f, Scal *s) {
+    template <class F> void pointwise(const F &f, Scal *s, cudaGraphConditionalHandle cond = 0) {
         cudaEvent_t e = tbeg(5, 0, (double)rw_words<F>() * N * sizeof(T), 0.0);
-        k_pointwise<F><<<(int)pw_blocks<F>(N), 256, 0, st>>>(N, f, partials, s);
+        k_pointwise<F><<<(int)pw_blocks<F>(N), 256, 0, st>>>(N, f, partials, s, cond);
         CK(cudaGetLastError());
         tend(e);
         ++launches;
@@ -1559,13 +1557,13 @@ struct Engine : EngineBase {
             auto iter_body = [&] {
                 x_fwd<NSx>(dir, sc);
                 spectral<NSx, NSx>(proj, sc, true);
-                x_inv<NSx>(eq, sc);
+                x_inv<NSx>(eq, sc, cap_cond);
             };
             if (batcher) {
                 MechLoop<NSx> q;
                 q.dir = dir; q.proj = proj; q.eq = eq;
                 batch_request(q);
-            } else if (run_loop(1, phi_in, nullptr, sc, iter_body)) {
+            } else if (run_loop(1, phi_in, nullptr, iter_body)) {
                 read_sc(sc);
                 count_loop(1, phi_in, nullptr, h_sc->iters);
             } else {
@@ -1642,13 +1640,13 @@ struct Engine : EngineBase {
             auto iter_body = [&] {
                 x_fwd<NSx>(dir, sc);
                 spectral<NSx, NSx>(proj, sc, true);
-                x_inv<NSx>(eq, sc);
+                x_inv<NSx>(eq, sc, cap_cond);
             };
             if (batcher) {
                 MechLoop<NSx> q;
                 q.dir = dir; q.proj = proj; q.eq = eq;
                 batch_request(q);
-            } else if (run_loop(1, phi_in, nullptr, sc, iter_body)) {
+            } else if (run_loop(1, phi_in, nullptr, iter_body)) {
                 read_sc(sc);
                 count_loop(1, phi_in, nullptr, h_sc->iters);
             } else {
@@ -1717,9 +1715,9 @@ struct Engine : EngineBase {
                 x_fwd<3>(dir, sc);
                 spectral<3, 3>(proj, sc, true);
                 x_inv<3>(eq, sc);
-                pointwise(up, sc);
+                pointwise(up, sc, cap_cond);
             };
-            if (run_loop(2, phi_in, nullptr, sc, iter_body)) {
+            if (run_loop(2, phi_in, nullptr, iter_body)) {
                 read_sc(sc);
                 count_loop(2, phi_in, nullptr, h_sc->iters);
             } else {
@@ -1789,13 +1787,13 @@ struct Engine : EngineBase {
                 spectral<1, Dx + 1>(pgrad, sc);
                 x_mid2<Dx + 1, Dx>(fluxu, sc);
                 spectral<Dx, 1>(divo, sc);
-                x_inv<1>(ew, sc);
+                x_inv<1>(ew, sc, cap_cond);
             };
             if (batcher) {
                 DmgLoop<Dx> q;
                 q.pdir = pdir; q.pgrad = pgrad; q.fluxu = fluxu; q.divo = divo; q.ew = ew;
                 batch_request(q);
-            } else if (run_loop(3, x, co.Ktab, sc, iter_body)) {
+            } else if (run_loop(3, x, co.Ktab, iter_body)) {
                 read_sc(sc);
                 count_loop(3, x, co.Ktab, h_sc->iters);
             } else {
@@ -2176,7 +2174,7 @@ struct Engine : EngineBase {
     // on the host (one read per reduction); the E components of the vectors too.
     T *nrbuf = nullptr;
     template <class F> void pointwise_n(const F &f, Scal *s, long long n) {
-        k_pointwise<F><<<(int)pw_blocks<F>(n), 256, 0, st>>>(n, f, partials, s);
+        k_pointwise<F><<<(int)pw_blocks<F>(n), 256, 0, st>>>(n, f, partials, s, 0);
         CK(cudaGetLastError());
         ++launches;
     }

@@ -733,15 +733,34 @@ __global__ void __launch_bounds__(x_max_threads<T>(), x_min_blocks<T>())
     x_fwd_body<T, NC>(g, RP, a.f, (C *)a.spec, tw, a.partials, a.sc);
 }
 
+// Condition of the while node whose body a kernel ends: set by the thread that has just updated the
+// solve's scalars (or by a kernel that skips because the solve is done), so that an iteration needs no
+// kernel of its own for it. 0: not in such a graph.
+__device__ __forceinline__ void loop_cond(cudaGraphConditionalHandle cond, const Scal *sc) {
+    if (cond) cudaGraphSetConditional(cond, sc->done ? 0u : 1u);
+}
+template <class F> struct FinCond {  // the finalizer of a reduction, then the loop condition
+    F fin;
+    cudaGraphConditionalHandle cond;
+    const Scal *sc;
+    __device__ void operator()(const double *t) const {
+        fin(t);
+        loop_cond(cond, sc);
+    }
+};
+
 // ---- x-axis inverse (c2r) pass with a fused epilogue --------------------------------------------
 template <typename T, int NC, class Epi>
 __device__ __forceinline__ void x_inv_body(const Geom &g, int RP, const typename cplx_of<T>::type *__restrict__ spec,
                                            const Epi &epi, const line_w<T> *__restrict__ tw, double *partials,
-                                           Scal *sc) {
+                                           Scal *sc, cudaGraphConditionalHandle cond) {
     typedef typename cplx_of<T>::type C;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C *s = reinterpret_cast<C *>(smem_raw);
-    if (epi.skip_if_done && sc->done) return;
+    if (epi.skip_if_done && sc->done) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) loop_cond(cond, sc);
+        return;
+    }
     const int nx = g.nx, LS = x_line_stride<T>(nx);
     const long long pair0 = (long long)blockIdx.x * RP;
     load_packed<T, NC>(g, spec, pair0, RP, s, LS);
@@ -783,14 +802,15 @@ __device__ __forceinline__ void x_inv_body(const Geom &g, int RP, const typename
 #pragma unroll
         for (int k = 0; k < NR1; ++k) acc[k] = (double)accf[k];
     }
-    if constexpr (Epi::NR > 0) reduce_finalize<Epi::NR>(acc, partials, sc, epi.fin(sc));
+    if constexpr (Epi::NR > 0)
+        reduce_finalize<Epi::NR>(acc, partials, sc, FinCond<typename Epi::Fin>{epi.fin(sc), cond, sc});
 }
 
 template <typename T, int NC, class Epi>
 __global__ void __launch_bounds__(x_inv_threads<T>(), sizeof(T) == 8 ? 2 : 1)
     k_x_inv(Geom g, int RP, const typename cplx_of<T>::type *__restrict__ spec, Epi epi,
-            const line_w<T> *__restrict__ tw, double *partials, Scal *sc) {
-    x_inv_body<T, NC>(g, RP, spec, epi, tw, partials, sc);
+            const line_w<T> *__restrict__ tw, double *partials, Scal *sc, cudaGraphConditionalHandle cond) {
+    x_inv_body<T, NC>(g, RP, spec, epi, tw, partials, sc, cond);
 }
 
 template <typename T, int NC, class Epi>
@@ -798,7 +818,7 @@ __global__ void __launch_bounds__(x_inv_threads<T>(), sizeof(T) == 8 ? 2 : 1)
     k_x_inv_b(Geom g, int RP, SlotArgs<Epi> args, const line_w<T> *__restrict__ tw) {
     typedef typename cplx_of<T>::type C;
     const SlotArg<Epi> &a = args.a[blockIdx.z];
-    x_inv_body<T, NC>(g, RP, (const C *)a.spec, a.f, tw, a.partials, a.sc);
+    x_inv_body<T, NC>(g, RP, (const C *)a.spec, a.f, tw, a.partials, a.sc, 0);
 }
 
 // ---- x-axis inverse, pointwise map, x-axis forward ----------------------------------------------
@@ -1025,14 +1045,19 @@ __global__ void __launch_bounds__(256) k_pointwise_b(long long N, SlotArgs<F> ar
 }
 
 template <class F>
-__global__ void __launch_bounds__(256) k_pointwise(long long N, F f, double *partials, Scal *sc) {
-    if (f.skip_if_done && sc->done) return;
+__global__ void __launch_bounds__(256) k_pointwise(long long N, F f, double *partials, Scal *sc,
+                                                   cudaGraphConditionalHandle cond) {
+    if (f.skip_if_done && sc->done) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) loop_cond(cond, sc);
+        return;
+    }
     double acc[F::NR > 0 ? F::NR : 1];
 #pragma unroll
     for (int k = 0; k < (F::NR > 0 ? F::NR : 1); ++k) acc[k] = 0.0;
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < N; v += stride) f.apply(v, acc);
-    if constexpr (F::NR > 0) reduce_finalize<F::NR>(acc, partials, sc, f.fin(sc), F::MAXRED);
+    if constexpr (F::NR > 0)
+        reduce_finalize<F::NR>(acc, partials, sc, FinCond<typename F::Fin>{f.fin(sc), cond, sc}, F::MAXRED);
 }
 
 }  // namespace pff

@@ -229,7 +229,7 @@ extern "C" int rve_dissipation_noalloc(int dim, const int n[3], double ell, int 
         const size_t sm = x_smem<double>(nx, xs.RP, 2);
         if (sm > 32 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         k<<<xs.blocks, xs.threads, sm, st>>>(g, xs.RP, spec, EpiDissChecked<2>{false, phi, Gc, A, gid, n_grains, ell}, twx,
-                                         partials, sc);
+                                         partials, sc, 0);
     } else {
         if (nz == 1) {
             // plate: xi_z = 0, so the gradient is taken in the y pass, as in 2D
@@ -249,7 +249,7 @@ extern "C" int rve_dissipation_noalloc(int dim, const int n[3], double ell, int 
         const size_t sm = x_smem<double>(nx, xs.RP, 3);
         if (sm > 32 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         k<<<xs.blocks, xs.threads, sm, st>>>(g, xs.RP, spec, EpiDissChecked<3>{false, phi, Gc, A, gid, n_grains, ell}, twx,
-                                         partials, sc);
+                                         partials, sc, 0);
     }
     if (cudaGetLastError() != cudaSuccess) return RVE_ECUDA;
     // D and Gamma were written to the scalar block by the last CTA; hand them to the caller.
