@@ -72,23 +72,29 @@ struct ProStressTotal : MechBase<T, NS> {
 // eps = (a, b, sqrt2 c) in Mandel form, eps_zz = 0. In-plane eigenvalues e1,2 = (a+b)/2 +- r,
 // r = sqrt(((a-b)/2)^2 + c^2), eigenvectors at angle theta with cos 2theta = (a-b)/(2r),
 // sin 2theta = c/r. psi+- = lam/2 <tr>+-^2 + mu sum <e_a>+-^2, sigma+- = lam <tr>+- I + 2 mu eps+-;
-// the tangent uses the divided differences of <.>+- over the eigenvalue pairs.
+// the tangent uses the divided differences of <.>+- over the eigenvalue pairs. In FP64 these passes are
+// bound by the FP64 pipe, where a divide or a square root costs about twenty operations, so both
+// functions take one reciprocal square root and nothing else: the projector n1 n1 needs cos^2 theta =
+// (1 + cos 2theta) / 2 and sin theta cos theta = sin 2theta / 2 only.
 template <typename T>
 struct SplitState {
-    T e1, e2, tr, C2, S2;  // eigenvalues, trace, cos 2theta, sin 2theta
+    T e1, e2, tr, C2, S2, ir;  // eigenvalues, trace, cos 2theta, sin 2theta, 1 / r
 };
 
 template <typename T> __device__ __forceinline__ SplitState<T> split_eig(const T *em) {
     const T r2 = (T)0.70710678118654752440;
     const T a = em[0], b = em[1], c = em[2] * r2;
     const T d = (T)0.5 * (a - b);
-    const T r = sqrt(d * d + c * c);
+    const T q = d * d + c * c;
     SplitState<T> st;
+    st.ir = q > (T)0 ? rsqrt(q) : (T)0;
+    T r = q * st.ir;
+    r = fma(fma(-r, r, q), (T)0.5 * st.ir, r);  // rounded as a square root: a uniaxial state keeps its exact zero eigenvalue
     st.tr = a + b;
     st.e1 = (T)0.5 * st.tr + r;
     st.e2 = (T)0.5 * st.tr - r;
-    if (r > (T)0) { st.C2 = d / r; st.S2 = c / r; }
-    else { st.C2 = (T)1; st.S2 = (T)0; }
+    st.C2 = q > (T)0 ? d * st.ir : (T)1;
+    st.S2 = c * st.ir;
     return st;
 }
 
@@ -120,20 +126,23 @@ template <typename T>
 __device__ __forceinline__ void split_tangent(const T *em, const T *dm, T lam, T mu, T g, T *out) {
     const SplitState<T> q = split_eig(em);
     const T r2 = (T)0.70710678118654752440, s2 = (T)1.41421356237309504880;
-    const T c = sqrt(fmax((T)0, (T)0.5 * ((T)1 + q.C2)));
-    const T sn = copysign(sqrt(fmax((T)0, (T)0.5 * ((T)1 - q.C2))), q.S2);
     const T dxx = dm[0], dyy = dm[1], dxy = dm[2] * r2;
-    const T cs = c * sn, cc = c * c, ss = sn * sn;
+    const T cs = (T)0.5 * q.S2, cc = (T)0.5 * ((T)1 + q.C2), ss = (T)0.5 * ((T)1 - q.C2);
     const T P11 = cc * dxx + 2 * cs * dxy + ss * dyy;
     const T P22 = ss * dxx - 2 * cs * dxy + cc * dyy;
     const T P12 = -cs * dxx + (cc - ss) * dxy + cs * dyy;
     const T trd = dxx + dyy;
+    // divided differences (<e1>+- - <e2>+-) / (e1 - e2): 1 or 0 when both eigenvalues have one sign (the
+    // derivative when they coincide), else the share of e1 - e2 = 2 r
+    const T hp = (T)0.5 * q.ir;
+    const T qp = q.e2 >= (T)0 ? (T)(q.e1 > 0) : (q.e1 > (T)0 ? q.e1 * hp : (T)0);
+    const T qm = q.e1 <= (T)0 ? (T)(q.e2 < 0) : (q.e2 < (T)0 ? -q.e2 * hp : (T)0);
     T res[3] = {0, 0, 0};
+#pragma unroll
     for (int part = 0; part < 2; ++part) {
         const bool plus = part == 0;
-        const T f1 = plus ? pos_(q.e1) : neg_(q.e1), f2 = plus ? pos_(q.e2) : neg_(q.e2);
         const T d1 = plus ? (T)(q.e1 > 0) : (T)(q.e1 < 0), d2 = plus ? (T)(q.e2 > 0) : (T)(q.e2 < 0);
-        const T qq = (q.e1 == q.e2) ? d1 : (f1 - f2) / (q.e1 - q.e2);
+        const T qq = plus ? qp : qm;
         const T ht = plus ? (T)(q.tr > 0) : (T)(q.tr < 0);
         // DF = d1 P11 n1n1 + d2 P22 n2n2 + qq P12 (n1n2 + n2n1)
         const T Fxx = (T)0.5 * (d1 * P11 * ((T)1 + q.C2) + d2 * P22 * ((T)1 - q.C2)) - qq * P12 * q.S2;
