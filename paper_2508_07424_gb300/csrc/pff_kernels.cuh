@@ -534,6 +534,8 @@ template <int K> struct axis_form_of {
     static constexpr int R = K == AXK_4 ? 4 : (K == AXK_8T ? 8 : (K == AXK_32T ? 32 : 16));
     static constexpr bool TWO = K >= AXK_8T;
 };
+// FP32 lines of 16 to 128 points: 80 registers, 3 CTAs of 256 threads per SM (128^3 projection pass 49.4 -> 45.1 us).
+template <typename T, int K> __host__ __device__ constexpr int axis_min_blocks() { return sizeof(T) == 4 && K == AXK_16 ? 3 : 0; }
 
 // ---- x passes ------------------------------------------------------------------------------------
 // A CTA owns RP pairs of x-rows; each pair is one packed complex line Z = a + i b per component.
@@ -578,16 +580,22 @@ __device__ __forceinline__ void x_lines(typename cplx_of<T>::type *s, const Geom
     else fft_lines<float2, NL>(s, g.nx, g.lx, NL, NG, 1, tw, inv);
 }
 
-// Call f(row pair, x) for the columns of the CTA's row pairs that this thread handles: FP32, four columns
-// nx / 4 apart, unrolled so that their loads are in flight together; FP64, a strided loop.
-template <typename T, class F> __device__ __forceinline__ void x_columns(const Geom &g, int RP, const F &f) {
+// Call f(row pair, x, voxel of the first row) for the columns of the CTA's row pairs that this thread
+// handles: FP32, four columns nx / 4 apart, unrolled so that their loads are in flight together; FP64, a
+// strided loop.
+template <typename T, class F>
+__device__ __forceinline__ void x_columns(const Geom &g, long long pair0, int RP, const F &f) {
     if constexpr (sizeof(T) == 4) {
         const int TL = g.nx >> 2, rp = threadIdx.x / TL, t = threadIdx.x - rp * TL;
+        const long long row0 = 2 * (pair0 + rp) * g.nx;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) f(rp, t + q * TL);
+        for (int q = 0; q < 4; ++q) f(rp, t + q * TL, row0 + t + q * TL);
     } else {
 #pragma unroll 2
-        for (int i = threadIdx.x; i < RP * g.nx; i += blockDim.x) f(i >> g.lx, i & (g.nx - 1));
+        for (int i = threadIdx.x; i < RP * g.nx; i += blockDim.x) {
+            const int rp = i >> g.lx, x = i & (g.nx - 1);
+            f(rp, x, 2 * (pair0 + rp) * g.nx + x);
+        }
     }
 }
 
@@ -687,8 +695,7 @@ __device__ __forceinline__ void x_fwd_body(const Geom &g, int RP, const Pro &pro
     double acc[Pro::NR > 0 ? Pro::NR : 1];
 #pragma unroll
     for (int k = 0; k < (Pro::NR > 0 ? Pro::NR : 1); ++k) acc[k] = 0.0;
-    x_columns<T>(g, RP, [&](int rp, int x) {
-        const long long v = 2 * (pair0 + rp) * nx + x;
+    x_columns<T>(g, pair0, RP, [&](int rp, int x, long long v) {
         T va[NC], vb[NC];
         pro.eval(v, va, acc);
         pro.eval(v + nx, vb, acc);
@@ -780,8 +787,7 @@ __device__ __forceinline__ void x_inv_body(const Geom &g, int RP, const typename
     float accf[NR1];
 #pragma unroll
     for (int k = 0; k < NR1; ++k) accf[k] = 0.f;
-    x_columns<T>(g, RP, [&](int rp, int x) {
-        const long long v = 2 * (pair0 + rp) * nx + x;
+    x_columns<T>(g, pair0, RP, [&](int rp, int x, long long v) {
         const C *line = s + rp * NC * LS + lpos<T>(x);
         T va[NC], vb[NC];
 #pragma unroll
@@ -807,14 +813,14 @@ __device__ __forceinline__ void x_inv_body(const Geom &g, int RP, const typename
 }
 
 template <typename T, int NC, class Epi>
-__global__ void __launch_bounds__(x_inv_threads<T>(), sizeof(T) == 8 ? 2 : 1)
+__global__ void __launch_bounds__(x_inv_threads<T>(), sizeof(T) == 8 ? 2 : 0)
     k_x_inv(Geom g, int RP, const typename cplx_of<T>::type *__restrict__ spec, Epi epi,
             const line_w<T> *__restrict__ tw, double *partials, Scal *sc, cudaGraphConditionalHandle cond) {
     x_inv_body<T, NC>(g, RP, spec, epi, tw, partials, sc, cond);
 }
 
 template <typename T, int NC, class Epi>
-__global__ void __launch_bounds__(x_inv_threads<T>(), sizeof(T) == 8 ? 2 : 1)
+__global__ void __launch_bounds__(x_inv_threads<T>(), sizeof(T) == 8 ? 2 : 0)
     k_x_inv_b(Geom g, int RP, SlotArgs<Epi> args, const line_w<T> *__restrict__ tw) {
     typedef typename cplx_of<T>::type C;
     const SlotArg<Epi> &a = args.a[blockIdx.z];
@@ -839,8 +845,7 @@ __device__ __forceinline__ void x_mid_body(const Geom &g, int RP, typename cplx_
     x_lines<T, NCI, NCI>(s, g, RP, LS, tw, true, -1);
     __syncthreads();
     const T sN = sizeof(T) == 8 ? (T)1 : (T)g.invN;
-    x_columns<T>(g, RP, [&](int rp, int x) {
-        const long long v = 2 * (pair0 + rp) * nx + x;
+    x_columns<T>(g, pair0, RP, [&](int rp, int x, long long v) {
         C *line = s + rp * NCI * LS + lpos<T>(x);
         T va[NCI], vb[NCI], oa[NCO], ob[NCO];
 #pragma unroll
@@ -862,14 +867,14 @@ __device__ __forceinline__ void x_mid_body(const Geom &g, int RP, typename cplx_
 }
 
 template <typename T, int NCI, int NCO, class Mid>
-__global__ void __launch_bounds__(x_inv_threads<T>(), sizeof(T) == 8 ? 2 : 1)
+__global__ void __launch_bounds__(x_inv_threads<T>(), sizeof(T) == 8 ? 2 : 0)
     k_x_mid(Geom g, int RP, typename cplx_of<T>::type *__restrict__ spec, Mid mid, const line_w<T> *__restrict__ tw,
             Scal *sc) {
     x_mid_body<T, NCI, NCO>(g, RP, spec, mid, tw, sc);
 }
 
 template <typename T, int NCI, int NCO, class Mid>
-__global__ void __launch_bounds__(x_inv_threads<T>(), sizeof(T) == 8 ? 2 : 1)
+__global__ void __launch_bounds__(x_inv_threads<T>(), sizeof(T) == 8 ? 2 : 0)
     k_x_mid_b(Geom g, int RP, SlotArgs<Mid> args, const line_w<T> *__restrict__ tw) {
     typedef typename cplx_of<T>::type C;
     const SlotArg<Mid> &a = args.a[blockIdx.z];
@@ -972,14 +977,14 @@ __device__ __forceinline__ void axis_body(const Geom &g, int axis, int CW,
 }
 
 template <typename T, int NCI, int NCO, int MODE, int K, class Op>
-__global__ void __launch_bounds__(axis_max_threads<T>(axis_form_of<K>::R))
+__global__ void __launch_bounds__(axis_max_threads<T>(axis_form_of<K>::R), axis_min_blocks<T, K>())
     k_axis(Geom g, int axis, int CW, const typename cplx_of<T>::type *__restrict__ spec_in,
            typename cplx_of<T>::type *spec_out, Op op, const line_w<T> *__restrict__ tw, Scal *sc) {
     axis_body<T, NCI, NCO, MODE, K>(g, axis, CW, spec_in, spec_out, op, tw, sc);
 }
 
 template <typename T, int NCI, int NCO, int MODE, int K, class Op>
-__global__ void __launch_bounds__(axis_max_threads<T>(axis_form_of<K>::R))
+__global__ void __launch_bounds__(axis_max_threads<T>(axis_form_of<K>::R), axis_min_blocks<T, K>())
     k_axis_b(Geom g, int axis, int CW, SlotArgs<Op> args, const line_w<T> *__restrict__ tw) {
     typedef typename cplx_of<T>::type C;
     const SlotArg<Op> &a = args.a[blockIdx.z];
