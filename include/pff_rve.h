@@ -329,8 +329,7 @@ int rve_server_destroy(rve_server s);
  * stderr; so do grids too small for one warp per x-pass CTA (as for rve_create). Extents are
  * powers of two from 4 to 1024; dim = 3 also takes plates one voxel thick (n[2] = 1), as
  * rve_create does.
- * The first call on a device looks up the array's device address (cudaGetSymbolAddress) and
- * copies a small table of FFT twiddles into the library's constant memory, so
+ * The first call on a device looks up the array's device address (cudaGetSymbolAddress), so
  * make that first call before any stream capture. All calls share the array: calls that
  * overlap on the GPU (different streams, different host threads) race and must be ordered by
  * the caller. Each call clears the parts of the array it relies on. */

@@ -9,7 +9,7 @@
 // in one file-scope __device__ array of fixed size that each GPU loading the library holds
 // until the process exits.
 //
-// The computation is the same three fused passes the engine uses for D and Gamma:
+// One launch sets up the call's tables; the computation is the same three fused passes the engine uses for D and Gamma:
 // the forward r2c FFT of phi, the spectral gradient i xi~ phi^ (frequency tables built in the
 // scratch array), and the inverse c2r FFT with
 // the reduction of sum Gc (phi^2/(2l) + l/2 grad phi . A grad phi).
@@ -49,35 +49,41 @@ static int cw_of(int L) {
     return cw;
 }
 
-// Frequencies xi~ = 2 pi k / n (FFT order, Nyquist set to zero) on one axis; the x axis covers
-// the padded half-spectrum columns, whose padding gets zero.
-__global__ void k_xi(double *xi, int n, int len, int half) {
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= len) return;
-    const int lim = half ? n / 2 + 1 : n;
+// Set-up of a call in one launch (latency is all there is to it: 8 separate launches and clears took
+// half of the call's 67 us at 128^2): the solver scalars (the reduction counter must start at zero; state
+// left by an earlier call is not trusted), the twiddles of the three axes in the fixed-point form of the
+// FP64 transforms, and the frequencies xi~ = 2 pi k / n (FFT order, Nyquist set to zero; the x axis covers
+// the padded half-spectrum columns, whose padding gets zero). The padding columns of the spectra are
+// not cleared: every column is transformed by itself and the inverse x pass reads none of them.
+__global__ void k_setup(Scal *sc, fxw *tw, double *xi, int nx, int ny, int nz, int Px) {
+    int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0) *sc = Scal{};
+    const int nt = nx + ny + nz;
+    if (i < nt) {
+        const int L = i < nx ? nx : (i < nx + ny ? ny : nz), m = i < nx ? i : (i < nx + ny ? i - nx : i - nx - ny);
+        double s, c;
+        sincospi(-2.0 * (double)m / (double)L, &s, &c);
+        auto put = [](double v, int &h, int &l) {
+            v *= 1073741824.0;
+            h = (int)rint(v);
+            l = (int)rint((v - (double)h) * 2147483648.0);
+        };
+        fxw w;
+        put(c, w.rh, w.rl);
+        put(s, w.ih, w.il);
+        tw[i] = w;
+        return;
+    }
+    i -= nt;
+    if (i >= Px + ny + nz) return;
+    const bool x = i < Px;
+    const int n = x ? nx : (i < Px + ny ? ny : nz), k = x ? i : (i < Px + ny ? i - Px : i - Px - ny);
     double v = 0.0;
-    if (k < lim && 2 * k != n) {
+    if (k < (x ? n / 2 + 1 : n) && 2 * k != n) {
         const int kk = k <= n / 2 ? k : k - n;
         v = 6.283185307179586476925286766559 * (double)kk / (double)n;
     }
-    xi[k] = v;
-}
-
-// Twiddles in the fixed-point form of the FP64 transforms.
-__global__ void k_twiddles(fxw *tw, int L) {
-    int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= L) return;
-    double s, c;
-    sincospi(-2.0 * (double)m / (double)L, &s, &c);
-    auto put = [](double v, int &h, int &l) {
-        v *= 1073741824.0;
-        h = (int)rint(v);
-        l = (int)rint((v - (double)h) * 2147483648.0);
-    };
-    fxw w;
-    put(c, w.rh, w.rl);
-    put(s, w.ih, w.il);
-    tw[m] = w;
+    xi[i] = v;
 }
 
 // Epilogue of the last pass: the dissipation density of Eq. (CrackLenght_ani) summed with and
@@ -93,6 +99,7 @@ struct EpiDissChecked {
     const int *gid;
     int n_grains;
     double ell;
+    double *result;  // D and Gamma, the caller's
     __device__ void apply(long long v, const double *gr, double *acc) const {
         const int gg = gid[v];
         if (gg < 0 || gg >= n_grains) {
@@ -116,10 +123,10 @@ struct EpiDissChecked {
         acc[1] += dens;
     }
     struct Fin {
-        Scal *sc;
-        __device__ void operator()(const double *t) const { sc->D = t[0]; sc->Gamma = t[1]; }
+        double *result;
+        __device__ void operator()(const double *t) const { result[0] = t[0]; result[1] = t[1]; }
     };
-    __device__ Fin fin(Scal *sc) const { return Fin{sc}; }
+    __device__ Fin fin(Scal *) const { return Fin{result}; }
 };
 
 }  // namespace pffnoalloc
@@ -191,45 +198,39 @@ extern "C" int rve_dissipation_noalloc(int dim, const int n[3], double ell, int 
     double2 *spec = (double2 *)(base + lay.spec);
     cudaStream_t st = (cudaStream_t)stream;
 
-    // state left by an earlier call is not trusted: reset the scalars (the reduction counter
-    // must start at zero) and the spectral buffer (its padding columns are read by the FFTs).
-    if (cudaMemsetAsync(sc, 0, sizeof(Scal), st) != cudaSuccess) return RVE_ECUDA;
-    if (cudaMemsetAsync(spec, 0, sizeof(double2) * (size_t)dim * (size_t)g.Nh, st) != cudaSuccess) return RVE_ECUDA;
-    k_twiddles<<<(nx + 255) / 256, 256, 0, st>>>(twx, nx);
-    k_twiddles<<<(ny + 255) / 256, 256, 0, st>>>(twy, ny);
-    if (nz > 1) k_twiddles<<<(nz + 255) / 256, 256, 0, st>>>(twz, nz);
-    k_xi<<<(g.Px + 255) / 256, 256, 0, st>>>(xix, nx, g.Px, 1);
-    k_xi<<<(ny + 255) / 256, 256, 0, st>>>(xiy, ny, ny, 0);
-    k_xi<<<(nz + 255) / 256, 256, 0, st>>>(xiz, nz, nz, 0);
-
+    {
+        const int n_el = (nx + ny + nz) + (g.Px + ny + nz);
+        k_setup<<<(n_el + 127) / 128, 128, 0, st>>>(sc, twx, xix, nx, ny, nz, g.Px);
+        if (cudaGetLastError() != cudaSuccess) return RVE_ECUDA;
+    }
+    auto launch = [&](auto kernel, dim3 grid, int threads, size_t sm, auto... args) -> cudaError_t {
+        if (sm > 32 * 1024) {
+            const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+            if (e != cudaSuccess) return e;
+        }
+        kernel<<<grid, threads, sm, st>>>(args...);
+        return cudaGetLastError();
+    };
     auto axis_launch = [&](auto kernel, int ax, int NM, const auto &op, const fxw *tw) -> cudaError_t {
         const int L = ax == 1 ? ny : nz;
         const int CW = ax == 1 ? cwy : cwz;
         int threads;
         size_t sm;
         axis_shape<double>(L, NM, CW, threads, sm);
-        if (sm > 32 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        kernel<<<dim3(g.Px / CW, ax == 1 ? nz : ny), threads, sm, st>>>(g, ax, CW, spec, spec, op, tw, sc);
-        return cudaGetLastError();
+        return launch(kernel, dim3(g.Px / CW, ax == 1 ? nz : ny), threads, sm, g, ax, CW, (const double2 *)spec, spec, op, tw, sc);
     };
-
     // forward x pass of phi
-    {
-        auto k = k_x_fwd<double, 1, ProField<double>>;
-        const size_t sm = x_smem<double>(nx, xs.RP, 1);
-        if (sm > 32 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        k<<<xs.blocks, xs.threads, sm, st>>>(g, xs.RP, ProField<double>{false, phi}, spec, twx, partials, sc);
-        if (cudaGetLastError() != cudaSuccess) return RVE_ECUDA;
-    }
+    if (launch(k_x_fwd<double, 1, ProField<double>>, dim3(xs.blocks), xs.threads, x_smem<double>(nx, xs.RP, 1), g, xs.RP,
+               ProField<double>{false, phi}, spec, (const fxw *)twx, partials, sc) != cudaSuccess)
+        return RVE_ECUDA;
     const int32_t *gid = grain_id;
     if (dim == 2) {
         if (axis_launch(axis_kernel<double, 1, 2, AX_FWD_OP_INV, OpGrad<double2, 2>>(ny), 1, 2, OpGrad<double2, 2>{false, xi}, twy))
             return RVE_ECUDA;
-        auto k = k_x_inv<double, 2, EpiDissChecked<2>>;
-        const size_t sm = x_smem<double>(nx, xs.RP, 2);
-        if (sm > 32 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        k<<<xs.blocks, xs.threads, sm, st>>>(g, xs.RP, spec, EpiDissChecked<2>{false, phi, Gc, A, gid, n_grains, ell}, twx,
-                                         partials, sc, 0);
+        if (launch(k_x_inv<double, 2, EpiDissChecked<2>>, dim3(xs.blocks), xs.threads, x_smem<double>(nx, xs.RP, 2), g,
+                   xs.RP, (const double2 *)spec, EpiDissChecked<2>{false, phi, Gc, A, gid, n_grains, ell, out},
+                   (const fxw *)twx, partials, sc, (cudaGraphConditionalHandle)0) != cudaSuccess)
+            return RVE_ECUDA;
     } else {
         if (nz == 1) {
             // plate: xi_z = 0, so the gradient is taken in the y pass, as in 2D
@@ -245,16 +246,10 @@ extern "C" int rve_dissipation_noalloc(int dim, const int n[3], double ell, int 
             if (axis_launch(axis_kernel<double, 3, 3, AX_INV, OpGrad<double2, 3>>(ny), 1, 3, OpGrad<double2, 3>{false, xi}, twy))
                 return RVE_ECUDA;
         }
-        auto k = k_x_inv<double, 3, EpiDissChecked<3>>;
-        const size_t sm = x_smem<double>(nx, xs.RP, 3);
-        if (sm > 32 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        k<<<xs.blocks, xs.threads, sm, st>>>(g, xs.RP, spec, EpiDissChecked<3>{false, phi, Gc, A, gid, n_grains, ell}, twx,
-                                         partials, sc, 0);
+        if (launch(k_x_inv<double, 3, EpiDissChecked<3>>, dim3(xs.blocks), xs.threads, x_smem<double>(nx, xs.RP, 3), g,
+                   xs.RP, (const double2 *)spec, EpiDissChecked<3>{false, phi, Gc, A, gid, n_grains, ell, out},
+                   (const fxw *)twx, partials, sc, (cudaGraphConditionalHandle)0) != cudaSuccess)
+            return RVE_ECUDA;
     }
-    if (cudaGetLastError() != cudaSuccess) return RVE_ECUDA;
-    // D and Gamma were written to the scalar block by the last CTA; hand them to the caller.
-    if (cudaMemcpyAsync(out, &sc->D, sizeof(double), cudaMemcpyDeviceToDevice, st) != cudaSuccess) return RVE_ECUDA;
-    if (cudaMemcpyAsync(out + 1, &sc->Gamma, sizeof(double), cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-        return RVE_ECUDA;
     return RVE_OK;
 }
