@@ -104,7 +104,17 @@ constexpr int kBadLine = 1 << 20;
 // imaginary parts. Converts to fixed point on the way in; on the way out back to FP64 scaled by
 // 2^-osh, or leaves integers with their e0 (fx_out) in the int array at ke0 when ke0 >= 0.
 // A function of its own, called once or twice per kernel, for the build time and because one
-// instance serves every length. Every thread of the CTA calls it; blockDim is a multiple of T.
+// instance serves every length. Every thread of the CTA calls it; blockDim is a multiple of T and of 32.
+// SOME: there may be warps without a line (x passes: three lines of 512 points for 256 threads). They
+// leave, and a line that spans several warps synchronises its own T threads by a named barrier (512^2
+// damage passes 18.7 / 30.7 -> 14.8 / 26.5 us). The column passes have a line for every thread; there
+// the CTA barrier is the faster one (36.6 against 38.2 us).
+template <bool SOME> __device__ __forceinline__ void line_sync(int lgT, int group) {
+    if (lgT <= 5) __syncwarp();
+    else if constexpr (SOME) asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "r"(1 << lgT) : "memory");
+    else __syncthreads();
+}
+template <bool SOME>
 static __device__ __noinline__ void fx_lines(int nlines, int LS, int lgL, const fxw *__restrict__ tw, bool inv, int osh,
                                              int ke0, int NL, int NG) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -112,9 +122,11 @@ static __device__ __noinline__ void fx_lines(int nlines, int LS, int lgL, const 
     __shared__ float wl1[32];
     const int lgT = lgL > 3 ? lgL - 3 : 0, TH = 1 << lgT;
     const int t = threadIdx.x & (TH - 1), gpc = blockDim.x >> lgT, nv = lgL < 3 ? 1 << lgL : 8;
-    const bool wide = TH > 32;  // a line spans several warps: CTA barriers
+    const bool wide = TH > 32;  // a line spans several warps
+    const int group = threadIdx.x >> lgT;  // at most 8 groups of more than a warp (512 threads)
     for (int first = 0; first < nlines; first += gpc) {
-        const int line = first + (threadIdx.x >> lgT);
+        if (SOME && first + ((int)(threadIdx.x & ~31u) >> lgT) >= nlines) break;  // no line in this warp
+        const int line = first + group;
         const bool valid = line < nlines;
         const int at = NL == NG ? line : line / NL * NG + line % NL;
         double2 *p = reinterpret_cast<double2 *>(smem_raw) + (valid ? at * LS : 0);
@@ -143,8 +155,8 @@ static __device__ __noinline__ void fx_lines(int nlines, int LS, int lgL, const 
                 wmx[threadIdx.x >> 5] = mx;
                 wl1[threadIdx.x >> 5] = l1;
             }
-            __syncthreads();
-            const int w0 = (threadIdx.x >> lgT) << (lgT - 5), nw = 1 << (lgT - 5);
+            line_sync<SOME>(lgT, group);
+            const int w0 = group << (lgT - 5), nw = 1 << (lgT - 5);
             for (int w = 0; w < nw; ++w) mx = max(mx, wmx[w0 + w]);
             l1 = 0.f;
             for (int w = 0; w < nw; ++w) {
@@ -166,14 +178,12 @@ static __device__ __noinline__ void fx_lines(int nlines, int LS, int lgL, const 
                 }
                 fx_dft8(v);
                 if (left == 3) break;
-                if (wide) __syncthreads();
-                else __syncwarp();
+                line_sync<SOME>(lgT, group);
                 if (valid) {
 #pragma unroll
                     for (int r = 0; r < 8; ++r) q[lpos<double>(((t - kk) << 3) + kk + (r << lgN))] = v[r];
                 }
-                if (wide) __syncthreads();
-                else __syncwarp();
+                line_sync<SOME>(lgT, group);
 #pragma unroll
                 for (int m = 0; m < 8; ++m) v[m] = q[lpos<double>(t + (m << lgT))];
                 lgN += 3;
@@ -576,7 +586,7 @@ template <typename T> __device__ __forceinline__ int x_ke0(int nlines, int LS) {
 template <typename T, int NL, int NG>
 __device__ __forceinline__ void x_lines(typename cplx_of<T>::type *s, const Geom &g, int RP, int LS,
                                         const line_w<T> *__restrict__ tw, bool inv, int ke0) {
-    if constexpr (sizeof(T) == 8) fx_lines(RP * NL, LS, g.lx, tw, inv, inv ? g.lx + g.ly + g.lz : 0, ke0, NL, NG);
+    if constexpr (sizeof(T) == 8) fx_lines<true>(RP * NL, LS, g.lx, tw, inv, inv ? g.lx + g.ly + g.lz : 0, ke0, NL, NG);
     else fft_lines<float2, NL>(s, g.nx, g.lx, NL, NG, 1, tw, inv);
 }
 
@@ -890,7 +900,7 @@ __global__ void __launch_bounds__(x_inv_threads<T>(), sizeof(T) == 8 ? 2 : 0)
 template <typename T, int K, bool INV>
 __device__ __forceinline__ void axis_lines(typename cplx_of<T>::type *s, int nlines, int LS, int lgL,
                                            const line_w<T> *__restrict__ tw) {
-    if constexpr (sizeof(T) == 8) fx_lines(nlines, LS, lgL, tw, INV, 0, -1, 1, 1);
+    if constexpr (sizeof(T) == 8) fx_lines<false>(nlines, LS, lgL, tw, INV, 0, -1, 1, 1);
     else warp_lines<float2, axis_form_of<K>::R, axis_form_of<K>::TWO, INV>(s, nlines, LS, 1 << lgL, tw);
 }
 
