@@ -558,7 +558,8 @@ template <typename T> __host__ __device__ constexpr int x_max_threads() { return
 template <typename T> __host__ __device__ constexpr int x_inv_threads() { return sizeof(T) == 8 ? 256 : 512; }
 template <typename T> __host__ __device__ constexpr int x_min_blocks() { return sizeof(T) == 8 ? 2 : 3; }
 
-// Launch shape. FP32: 128 threads of 4 columns. FP64: 256 columns (256 threads from 512 columns on); on
+// Launch shape. FP32: 128 threads of 4 columns. FP64: 256 columns, a thread per column up to 256 (half the
+// threads left 7 warps per SM and two rounds of lines: 64x64x32 CG passes 35.1 / 28.3 -> 31.1 / 23.4 us); on
 // small grids an FP64 pass is bound by the FP64 work of the few SMs that hold a CTA, so there a CTA
 // takes as few row pairs as give a whole warp, until there are two CTAs per SM (64^2 with the
 // split: 4 -> 32 CTAs, 66 -> 24 us per forward pass; FP32 passes gained nothing from it).
@@ -572,7 +573,7 @@ template <typename T> inline XShape x_shape(int nx, long long pairs) {
     XShape x;
     x.RP = RP;
     x.blocks = (int)(pairs / RP);
-    x.threads = !fx ? RP * unit : (RP * nx >= 512 || x.blocks < 304 ? std::min(256, RP * nx) : std::max(32, RP * nx / 2));
+    x.threads = !fx ? RP * unit : std::max(32, std::min(256, RP * nx));
     return x;
 }
 // Dynamic shared memory: the lines, then (FP64) one exponent per line.
