@@ -550,13 +550,14 @@ template <typename T, int K> __host__ __device__ constexpr int axis_min_blocks()
 // ---- x passes ------------------------------------------------------------------------------------
 // A CTA owns RP pairs of x-rows; each pair is one packed complex line Z = a + i b per component.
 // Pointwise work runs over the RP nx columns of the pairs with every thread. Launch bounds: 256 threads,
-// 512 for the inverse and middle FP32 passes as before; on the FP32 forward path at least 3 CTAs of 256
-// threads per SM (<= 85 registers), so that more warps cover the latency of the fused prologue's loads,
-// which bound it on large grids (128^3: 174 -> 150 us per CG launch; the inverse and middle x
-// passes measured 5-10 % slower with the same bound and keep theirs).
+// 512 for the inverse and middle FP32 passes. The FP32 forward pass is bound by the latency of the
+// fused prologue's loads, so its registers are bounded for occupancy: 4 CTAs of 256 threads per SM up to
+// three components (64 registers: the 512 CTAs of a 1024^2 pass fit the 608 slots in one wave, 43.6 -> 31.8 us
+// per CG launch), 3 with six (80 registers; 128^3: 174 -> 150 us). The inverse and middle passes measured
+// 5-10 % slower with such a bound.
 template <typename T> __host__ __device__ constexpr int x_max_threads() { return 256; }
 template <typename T> __host__ __device__ constexpr int x_inv_threads() { return sizeof(T) == 8 ? 256 : 512; }
-template <typename T> __host__ __device__ constexpr int x_min_blocks() { return sizeof(T) == 8 ? 2 : 3; }
+template <typename T, int NC> __host__ __device__ constexpr int x_min_blocks() { return sizeof(T) == 8 ? 2 : (NC <= 3 ? 4 : 3); }
 
 // Launch shape. FP32: 128 threads of 4 columns. FP64: 256 columns, a thread per column up to 256 (half the
 // threads left 7 warps per SM and two rounds of lines: 64x64x32 CG passes 35.1 / 28.3 -> 31.1 / 23.4 us); on
@@ -723,7 +724,7 @@ __device__ __forceinline__ void x_fwd_body(const Geom &g, int RP, const Pro &pro
 }
 
 template <typename T, int NC, class Pro>
-__global__ void __launch_bounds__(x_max_threads<T>(), x_min_blocks<T>())
+__global__ void __launch_bounds__(x_max_threads<T>(), x_min_blocks<T, NC>())
     k_x_fwd(Geom g, int RP, Pro pro, typename cplx_of<T>::type *__restrict__ spec, const line_w<T> *__restrict__ tw,
             double *partials, Scal *sc) {
     x_fwd_body<T, NC>(g, RP, pro, spec, tw, partials, sc);
@@ -744,7 +745,7 @@ template <class F> struct SlotArgs {
 };
 
 template <typename T, int NC, class Pro>
-__global__ void __launch_bounds__(x_max_threads<T>(), x_min_blocks<T>())
+__global__ void __launch_bounds__(x_max_threads<T>(), x_min_blocks<T, NC>())
     k_x_fwd_b(Geom g, int RP, SlotArgs<Pro> args, const line_w<T> *__restrict__ tw) {
     typedef typename cplx_of<T>::type C;
     const SlotArg<Pro> &a = args.a[blockIdx.z];
