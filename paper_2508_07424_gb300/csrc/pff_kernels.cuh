@@ -549,15 +549,14 @@ template <typename T, int K> __host__ __device__ constexpr int axis_min_blocks()
 
 // ---- x passes ------------------------------------------------------------------------------------
 // A CTA owns RP pairs of x-rows; each pair is one packed complex line Z = a + i b per component.
-// Pointwise work runs over the RP nx columns of the pairs with every thread. Launch bounds: 256 threads,
-// 512 for the inverse and middle FP32 passes. The FP32 forward pass is bound by the latency of the
-// fused prologue's loads, so its registers are bounded for occupancy: 4 CTAs of 256 threads per SM up to
-// three components (64 registers: the 512 CTAs of a 1024^2 pass fit the 608 slots in one wave, 43.6 -> 31.8 us
-// per CG launch), 3 with six (80 registers; 128^3: 174 -> 150 us). The inverse and middle passes measured
-// 5-10 % slower with such a bound.
-template <typename T> __host__ __device__ constexpr int x_max_threads() { return 256; }
-template <typename T> __host__ __device__ constexpr int x_inv_threads() { return sizeof(T) == 8 ? 256 : 512; }
-template <typename T, int NC> __host__ __device__ constexpr int x_min_blocks() { return sizeof(T) == 8 ? 2 : (NC <= 3 ? 4 : 3); }
+// Pointwise work runs over the RP nx columns of the pairs with every thread, at most 256. The FP32
+// passes are bound by the latency of their loads, so the registers of the forward and inverse passes are
+// bounded for occupancy: 64 up to three components (the 512 CTAs of 256 threads of a 1024^2 pass fit the 608
+// slots in one wave instead of two, 43.6 -> 31.8 us per CG forward launch), 72 with six (the 2048 CTAs of
+// 128 threads of a 128^3 pass in two waves instead of three: CG forward 154 -> 131 us, inverse
+// 66 -> 59 us; 85 registers gain no wave and measured 5-10 % slower). FP64: two CTAs per SM.
+template <typename T, int NC> __host__ __device__ constexpr int x_max_regs() { return sizeof(T) == 8 ? 128 : (NC <= 3 ? 64 : 72); }
+template <typename T> __host__ __device__ constexpr int x_mid_threads() { return sizeof(T) == 8 ? 256 : 512; }
 
 // Launch shape. FP32: 128 threads of 4 columns. FP64: 256 columns, a thread per column up to 256 (half the
 // threads left 7 warps per SM and two rounds of lines: 64x64x32 CG passes 35.1 / 28.3 -> 31.1 / 23.4 us); on
@@ -724,7 +723,7 @@ __device__ __forceinline__ void x_fwd_body(const Geom &g, int RP, const Pro &pro
 }
 
 template <typename T, int NC, class Pro>
-__global__ void __launch_bounds__(x_max_threads<T>(), x_min_blocks<T, NC>())
+__global__ void __maxnreg__((x_max_regs<T, NC>()))
     k_x_fwd(Geom g, int RP, Pro pro, typename cplx_of<T>::type *__restrict__ spec, const line_w<T> *__restrict__ tw,
             double *partials, Scal *sc) {
     x_fwd_body<T, NC>(g, RP, pro, spec, tw, partials, sc);
@@ -745,7 +744,7 @@ template <class F> struct SlotArgs {
 };
 
 template <typename T, int NC, class Pro>
-__global__ void __launch_bounds__(x_max_threads<T>(), x_min_blocks<T, NC>())
+__global__ void __maxnreg__((x_max_regs<T, NC>()))
     k_x_fwd_b(Geom g, int RP, SlotArgs<Pro> args, const line_w<T> *__restrict__ tw) {
     typedef typename cplx_of<T>::type C;
     const SlotArg<Pro> &a = args.a[blockIdx.z];
@@ -825,14 +824,14 @@ __device__ __forceinline__ void x_inv_body(const Geom &g, int RP, const typename
 }
 
 template <typename T, int NC, class Epi>
-__global__ void __launch_bounds__(x_inv_threads<T>(), sizeof(T) == 8 ? 2 : 0)
+__global__ void __maxnreg__((x_max_regs<T, NC>()))
     k_x_inv(Geom g, int RP, const typename cplx_of<T>::type *__restrict__ spec, Epi epi,
             const line_w<T> *__restrict__ tw, double *partials, Scal *sc, cudaGraphConditionalHandle cond) {
     x_inv_body<T, NC>(g, RP, spec, epi, tw, partials, sc, cond);
 }
 
 template <typename T, int NC, class Epi>
-__global__ void __launch_bounds__(x_inv_threads<T>(), sizeof(T) == 8 ? 2 : 0)
+__global__ void __maxnreg__((x_max_regs<T, NC>()))
     k_x_inv_b(Geom g, int RP, SlotArgs<Epi> args, const line_w<T> *__restrict__ tw) {
     typedef typename cplx_of<T>::type C;
     const SlotArg<Epi> &a = args.a[blockIdx.z];
@@ -879,14 +878,14 @@ __device__ __forceinline__ void x_mid_body(const Geom &g, int RP, typename cplx_
 }
 
 template <typename T, int NCI, int NCO, class Mid>
-__global__ void __launch_bounds__(x_inv_threads<T>(), sizeof(T) == 8 ? 2 : 0)
+__global__ void __launch_bounds__(x_mid_threads<T>(), sizeof(T) == 8 ? 2 : 0)
     k_x_mid(Geom g, int RP, typename cplx_of<T>::type *__restrict__ spec, Mid mid, const line_w<T> *__restrict__ tw,
             Scal *sc) {
     x_mid_body<T, NCI, NCO>(g, RP, spec, mid, tw, sc);
 }
 
 template <typename T, int NCI, int NCO, class Mid>
-__global__ void __launch_bounds__(x_inv_threads<T>(), sizeof(T) == 8 ? 2 : 0)
+__global__ void __launch_bounds__(x_mid_threads<T>(), sizeof(T) == 8 ? 2 : 0)
     k_x_mid_b(Geom g, int RP, SlotArgs<Mid> args, const line_w<T> *__restrict__ tw) {
     typedef typename cplx_of<T>::type C;
     const SlotArg<Mid> &a = args.a[blockIdx.z];
