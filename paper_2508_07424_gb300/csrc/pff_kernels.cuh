@@ -494,15 +494,24 @@ __device__ __forceinline__ void wfft2_inv(C (&v)[R], C *line, int l, int L, cons
 
 // Transform the lines [0, nlines) of the tile, one line per lane group of S lanes, looping over
 // groups of lines when there are more lines than warps. INV selects the inverse network.
+// Lines of a tile of CW columns start 16 / CW elements apart modulo the 16 elements of a shared-memory
+// phase. The 16 / S lines that a half-warp works on together are taken dist = S CW / 16 apart, so that
+// they start S elements apart and their accesses fall on distinct banks (adjacent lines overlapped:
+// two-way conflicts on 128 points; 128^3 projection pass 45.2 -> 43.3 us).
 template <typename C, int R, bool TWO, bool INV>
-__device__ __forceinline__ void warp_lines(C *s, int nlines, int LS, int L, const C *__restrict__ tw) {
+__device__ __forceinline__ void warp_lines(C *s, int nlines, int LS, int L, int lgCW, const C *__restrict__ tw) {
     const int lgS = ilog2(L) - log2_of<R>::v, S = 1 << lgS;
     const int lpw = 32 >> lgS;  // lines per warp
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
     const int l = lane & (S - 1);
     for (int grp = warp; grp * lpw < nlines; grp += nwarps) {  // uniform across the warp
-        const int line = grp * lpw + (lane >> lgS);
+        int line = grp * lpw + (lane >> lgS);
         const bool valid = line < nlines;
+        const int lgd = lgS + lgCW - 4;  // log2 dist
+        if (!TWO && lgS < 4 && lgd > 0) {
+            const int r = line & ((1 << lgCW) - 1);
+            line = line - r + ((r & ((1 << (4 - lgS)) - 1)) << lgd) + (r >> (4 - lgS));
+        }
         C *p = s + (size_t)(valid ? line : 0) * LS;
         C v[R];
 #pragma unroll
@@ -899,10 +908,10 @@ __global__ void __launch_bounds__(x_mid_threads<T>(), sizeof(T) == 8 ? 2 : 0)
 // The tile is read from global memory with consecutive threads on consecutive kx (coalesced runs
 // of CW complex values per row) into shared memory, one line of L points per (component, column).
 template <typename T, int K, bool INV>
-__device__ __forceinline__ void axis_lines(typename cplx_of<T>::type *s, int nlines, int LS, int lgL,
+__device__ __forceinline__ void axis_lines(typename cplx_of<T>::type *s, int nlines, int LS, int lgL, int lgCW,
                                            const line_w<T> *__restrict__ tw) {
     if constexpr (sizeof(T) == 8) fx_lines<false>(nlines, LS, lgL, tw, INV, 0, -1, 1, 1);
-    else warp_lines<float2, axis_form_of<K>::R, axis_form_of<K>::TWO, INV>(s, nlines, LS, 1 << lgL, tw);
+    else warp_lines<float2, axis_form_of<K>::R, axis_form_of<K>::TWO, INV>(s, nlines, LS, 1 << lgL, lgCW, tw);
 }
 
 template <typename T, int NCI, int NCO, int MODE, int K, class Op>
@@ -958,7 +967,7 @@ __device__ __forceinline__ void axis_body(const Geom &g, int axis, int CW,
     }
     __syncthreads();
     // 2. transforms (and the operator between them)
-    axis_lines<T, K, MODE == AX_INV>(s, NCI * CW, LS, lgL, tw);
+    axis_lines<T, K, MODE == AX_INV>(s, NCI * CW, LS, lgL, lgCW, tw);
     if constexpr (MODE == AX_FWD_OP_INV) {
         __syncthreads();
         for (int i = threadIdx.x; i < npt; i += nth) {
@@ -975,7 +984,7 @@ __device__ __forceinline__ void axis_body(const Geom &g, int axis, int CW,
             for (int c = 0; c < NCO; ++c) s[((c << lgCW) + cc) * LS + lpos<T>(p)] = out[c];
         }
         __syncthreads();
-        axis_lines<T, K, true>(s, NCO * CW, LS, lgL, tw);
+        axis_lines<T, K, true>(s, NCO * CW, LS, lgL, lgCW, tw);
     }
     __syncthreads();
     // 3. coalesced store
