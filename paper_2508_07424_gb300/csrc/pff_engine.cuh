@@ -1176,13 +1176,10 @@ struct Engine : EngineBase {
         carveout_set.insert((const void *)kernel);
     }
     template <typename K> void prep_smem(K kernel, size_t bytes) {
-        const void *key = (const void *)kernel;
-        auto it = smem_set.find(key);
-        // opt in above 32 KB: static shared memory (reduction scratch) adds to the dynamic size
-        if (bytes > 32 * 1024 && (it == smem_set.end() || it->second < bytes)) {
-            CK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-            smem_set[key] = bytes;
-        }
+        size_t &known = smem_set[(const void *)kernel];  // this handle's view: never above what is set
+        if (known >= bytes) return;
+        CK(smem_raise(kernel, bytes));
+        known = bytes;
     }
     // Events around one launch while timing is on (returns the end event to record after it).
     cudaEvent_t tbeg(int kind, int sub, double bytes, double flops) {

@@ -74,3 +74,21 @@ def test_non_finite_values_reach_the_result(bad):
 
 def test_zero_field():
     assert (_library(np.zeros((1, 32, 32)), (32, 32, 1), 2, 2.0) == 0.0).all()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32r"])
+def test_a_smaller_grid_does_not_take_shared_memory_from_a_larger_one(monkeypatch, precision):
+    """The shared-memory opt-in belongs to the kernel, which serves every line length: a handle of 512-point
+    columns (37 KB in FP64) used between two calls of one of 1024-point columns (74 KB)."""
+    import synth
+    from paper_2508_07424_gb300 import build
+    from paper_2508_07424_gb300.rve import Rve
+    build.build()
+    monkeypatch.setenv("PFF_TILE_CW", "2")
+    rng = np.random.default_rng(1)
+    out = {}
+    hs = {ny: Rve.from_workload(synth.Workload(synth.homogeneous((64, ny)), ell=2.0, precision=precision)) for ny in (1024, 512)}
+    phi = {ny: rng.uniform(0.0, 1.0, (1, ny, 64)) for ny in hs}
+    for ny in (1024, 512, 1024):
+        got = hs[ny].dissipation(phi[ny]), hs[ny].mech_solve()
+        assert out.setdefault(ny, got)[0] == got[0]
