@@ -83,13 +83,14 @@ __device__ __forceinline__ int fx_scale(unsigned mx, float l1) {
     return 61 - (fl + (int)(mx >> 20) - 1023 - 63);
 }
 // d 2^k rounded to an integer. The mantissa sits at bits 10..62 and is shifted down by
-// 1085 - e - k >= 1 bits.
+// 1085 - e - k >= 1 bits, at most 64: from there on the value is below half a unit and (m >> 63) + 1 rounds to
+// zero (at 63 it would give one unit to every value however small, and the tails of a line would add up).
 __device__ __forceinline__ long long fx_in(double d, int k) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(d);
     const int hi = (int)(b >> 32);
     const int e = (hi >> 20) & 0x7ff;
     int s = 1085 - e - k;
-    s = s < 63 ? s : 63;
+    s = s < 64 ? s : 64;
     const unsigned long long m = (((b & 0xfffffffffffffull) | 0x10000000000000ull) << 10);
     unsigned long long u = (m >> (s - 1)) + 1;
     u >>= 1;
