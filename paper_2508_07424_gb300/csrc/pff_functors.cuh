@@ -133,10 +133,11 @@ __device__ __forceinline__ void split_tangent(const T *em, const T *dm, T lam, T
     const T P12 = -cs * dxx + (cc - ss) * dxy + cs * dyy;
     const T trd = dxx + dyy;
     // divided differences (<e1>+- - <e2>+-) / (e1 - e2): 1 or 0 when both eigenvalues have one sign (the
-    // derivative when they coincide), else the share of e1 - e2 = 2 r
+    // derivative when they coincide), else the share of e1 - e2 = 2 r. Neither test of the first two holds for
+    // a NaN, which then reaches the result: the stress above maps it to zero, so the solve would not see it
     const T hp = (T)0.5 * q.ir;
-    const T qp = q.e2 >= (T)0 ? (T)(q.e1 > 0) : (q.e1 > (T)0 ? q.e1 * hp : (T)0);
-    const T qm = q.e1 <= (T)0 ? (T)(q.e2 < 0) : (q.e2 < (T)0 ? -q.e2 * hp : (T)0);
+    const T qp = q.e2 >= (T)0 ? (T)(q.e1 > 0) : (q.e1 <= (T)0 ? (T)0 : q.e1 * hp);
+    const T qm = q.e1 <= (T)0 ? (T)(q.e2 < 0) : (q.e2 >= (T)0 ? (T)0 : -q.e2 * hp);
     T res[3] = {0, 0, 0};
 #pragma unroll
     for (int part = 0; part < 2; ++part) {
