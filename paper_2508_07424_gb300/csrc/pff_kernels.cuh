@@ -86,33 +86,6 @@ template <typename T> __host__ __device__ constexpr int x_line_stride(int L) {
 }
 
 
-// 4- and 8-point DFTs, natural order in and out (forward).
-__device__ __forceinline__ void fx_dft4(fx2 &a, fx2 &b, fx2 &c, fx2 &d) {
-    const fx2 p = cadd(a, c), m = csub(a, c), q = cadd(b, d), r = csub(b, d);
-    a = cadd(p, q);
-    b.x = m.x + r.y; b.y = m.y - r.x;
-    c = csub(p, q);
-    d.x = m.x - r.y; d.y = m.y + r.x;
-}
-__device__ __forceinline__ void fx_dft8(fx2 (&v)[8]) {
-    fx2 e[4], o[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        e[j] = cadd(v[j], v[j + 4]);
-        o[j] = csub(v[j], v[j + 4]);
-    }
-    // odd outputs: o_j w_8^j, w_8 = (1 - i) / sqrt 2 (the scaling before the sums: no fixed-point overflow)
-    const long long x1 = fx_mul_r2(o[1].x), y1 = fx_mul_r2(o[1].y), x3 = fx_mul_r2(o[3].x), y3 = fx_mul_r2(o[3].y);
-    o[1].x = x1 + y1; o[1].y = y1 - x1;
-    const fx2 t = o[2];
-    o[2].x = t.y; o[2].y = -t.x;
-    o[3].x = y3 - x3; o[3].y = -x3 - y3;
-    fx_dft4(e[0], e[1], e[2], e[3]);
-    fx_dft4(o[0], o[1], o[2], o[3]);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) { v[2 * j] = e[j]; v[2 * j + 1] = o[j]; }
-}
-
 // e0 of a line that holds an infinity or a NaN, or whose norm leaves the FP64 range.
 constexpr int kBadLine = 1 << 20;
 
@@ -141,7 +114,7 @@ static __device__ __noinline__ void fx_lines(int nlines, int LS, int lgL, const 
                                              int ke0, int NL, int NG) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ unsigned wmx[32];
-    __shared__ float wl1[32];
+    __shared__ float wnorm[32];
     const int lgT = lgL > 3 ? lgL - 3 : 0, TH = 1 << lgT;
     const int t = threadIdx.x & (TH - 1), gpc = blockDim.x >> lgT, nv = lgL < 3 ? 1 << lgL : 8;
     const bool wide = TH > 32;  // a line spans several warps
@@ -161,76 +134,45 @@ static __device__ __noinline__ void fx_lines(int nlines, int LS, int lgL, const 
             if (valid && m < nv) z = p[lpos<double>(t + (m << lgT))];
             d[m] = inv ? make_double2(z.y, z.x) : z;
         }
-        // scale of the line, from its largest value and its L1 norm
+        // scale of the line, from its largest value and a bound of its norm
         unsigned mx = 0;
 #pragma unroll
         for (int m = 0; m < 8; ++m) mx = max(mx, max(fx_hi_abs(d[m].x), fx_hi_abs(d[m].y)));
         const int sw = wide ? 32 : TH;
         for (int o = sw >> 1; o; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        const unsigned base = fx_l1_base(mx);
-        float l1 = 0.f;
+        const unsigned base = fx_norm_base(mx);
+        float norm = 0.f;
 #pragma unroll
-        for (int m = 0; m < 8; ++m) l1 += fx_l1_term(fx_hi_abs(d[m].x), base) + fx_l1_term(fx_hi_abs(d[m].y), base);
-        for (int o = sw >> 1; o; o >>= 1) l1 += __shfl_xor_sync(0xffffffffu, l1, o);
+        for (int m = 0; m < 8; ++m) norm += fx_norm_term(fx_hi_abs(d[m].x), fx_hi_abs(d[m].y), base);
+        for (int o = sw >> 1; o; o >>= 1) norm += __shfl_xor_sync(0xffffffffu, norm, o);
         if (wide) {
             if ((threadIdx.x & 31) == 0) {
                 wmx[threadIdx.x >> 5] = mx;
-                wl1[threadIdx.x >> 5] = l1;
+                wnorm[threadIdx.x >> 5] = norm;
             }
             line_sync<SOME>(lgT, group);
             const int w0 = group << (lgT - 5), nw = 1 << (lgT - 5);
             for (int w = 0; w < nw; ++w) mx = max(mx, wmx[w0 + w]);
-            l1 = 0.f;
+            norm = 0.f;
             for (int w = 0; w < nw; ++w) {
                 const int dE = (int)(mx >> 20) - (int)(wmx[w0 + w] >> 20);
-                l1 += dE < 126 ? wl1[w0 + w] * __int_as_float((127 - dE) << 23) : 0.f;
+                norm += dE < 126 ? wnorm[w0 + w] * __int_as_float((127 - dE) << 23) : 0.f;
             }
         }
-        const int k = fx_scale(mx, l1);
+        const int k = fx_scale(mx, norm);
         const int e0 = mx >= 0x7ff00000u || k <= -963 ? kBadLine : 1086 - k;
 #pragma unroll
         for (int m = 0; m < 8; ++m) v[m] = fx2{fx_in(d[m].x, k), fx_in(d[m].y, k)};
-        for (int lgN = 0;;) {  // self-sorting passes; Ns = 2^lgN sub-transform points done
-            const int left = lgL - lgN;
-            if (left >= 3) {
-                const int kk = t & ((1 << lgN) - 1);
-                if (lgN > 0) {
+        for (int lgN = 0; !fx_pass(v, lgL, lgT, lgN, t, tw); lgN += 3) {
+            const int at8 = fx_pass_out(lgN, t);
+            line_sync<SOME>(lgT, group);
+            if (valid) {
 #pragma unroll
-                    for (int r = 1; r < 8; ++r) v[r] = cmul(v[r], tw[(r * kk) << (left - 3)]);
-                }
-                fx_dft8(v);
-                if (left == 3) break;
-                line_sync<SOME>(lgT, group);
-                if (valid) {
-#pragma unroll
-                    for (int r = 0; r < 8; ++r) q[lpos<double>(((t - kk) << 3) + kk + (r << lgN))] = v[r];
-                }
-                line_sync<SOME>(lgT, group);
-#pragma unroll
-                for (int m = 0; m < 8; ++m) v[m] = q[lpos<double>(t + (m << lgT))];
-                lgN += 3;
-            } else if (left == 2) {
-                if (lgL == 2) {
-                    fx_dft4(v[0], v[1], v[2], v[3]);
-                } else {
-#pragma unroll
-                    for (int b = 0; b < 2; ++b) {
-                        const int j = t + (b << lgT);
-#pragma unroll
-                        for (int r = 1; r < 4; ++r) v[b + 2 * r] = cmul(v[b + 2 * r], tw[r * j]);
-                        fx_dft4(v[b], v[b + 2], v[b + 4], v[b + 6]);
-                    }
-                }
-                break;
-            } else {
-#pragma unroll
-                for (int b = 0; b < 4; ++b) {
-                    const fx2 c = cmul(v[b + 4], tw[t + (b << lgT)]);
-                    v[b + 4] = csub(v[b], c);
-                    v[b] = cadd(v[b], c);
-                }
-                break;
+                for (int r = 0; r < 8; ++r) q[lpos<double>(at8 + (r << lgN))] = v[r];
             }
+            line_sync<SOME>(lgT, group);
+#pragma unroll
+            for (int m = 0; m < 8; ++m) v[m] = q[lpos<double>(t + (m << lgT))];
         }
         if (valid) {
             if (ke0 >= 0) {
@@ -671,8 +613,8 @@ __device__ __forceinline__ void store_split(const Geom &g, typename cplx_of<T>::
             const int e0 = ke[at];
             for (int k = k0; k <= h; k += h) {  // k0 = 0 also stores the Nyquist column
                 const fx2 Z = line[lpos<T>(k)], Zm = line[lpos<T>((nx - k) & (nx - 1))];
-                C Xa = make_double2(fx_out(Z.x + Zm.x, e0 - 1), fx_out(Z.y - Zm.y, e0 - 1));
-                C Xb = make_double2(fx_out(Z.y + Zm.y, e0 - 1), fx_out(Zm.x - Z.x, e0 - 1));
+                C Xa = make_double2(fx_out_sum(Z.x, Zm.x, e0 - 1), fx_out_sum(Z.y, -Zm.y, e0 - 1));
+                C Xb = make_double2(fx_out_sum(Z.y, Zm.y, e0 - 1), fx_out_sum(Zm.x, -Z.x, e0 - 1));
                 if (e0 == kBadLine) Xa.x = Xa.y = Xb.x = Xb.y = fx_nan();
                 dst[k] = Xa;
                 dst[g.Px + k] = Xb;

@@ -66,7 +66,7 @@ __global__ void k_setup(Scal *sc, fxw *tw, double *xi, int nx, int ny, int nz, i
         auto put = [](double v, int &h, int &l) {
             v *= 1073741824.0;
             h = (int)rint(v);
-            l = (int)rint((v - (double)h) * 2147483648.0);
+            l = (int)fmin(fmax(rint((v - (double)h) * 4294967296.0), -2147483647.0), 2147483647.0);
         };
         fxw w;
         put(c, w.rh, w.rl);
