@@ -40,6 +40,7 @@
 #include "pff_batch.cuh"
 #include "pff_common.cuh"
 #include "pff_functors.cuh"
+#include "pff_host.cuh"
 #include "pff_kernels.cuh"
 #include "pff_newton.cuh"
 
@@ -2707,11 +2708,7 @@ struct Engine : EngineBase {
         }
         default: return RVE_EINVAL;
         }
-        // Touch the caller's pages while the conversion runs: the device copies straight into pageable memory
-        // here, and pages that are not mapped yet (a fresh 25 MB numpy array) are faulted in from its side:
-        // 0.2 ms for mapped pages, up to 20 ms for fresh ones, 1.1 ms for fresh ones touched first
-        for (size_t i = 0; i < n; i += 4096 / sizeof(double)) reinterpret_cast<volatile double *>(host)[i] = 0.0;
-        if (n) reinterpret_cast<volatile double *>(host)[n - 1] = 0.0;
+        map_pages(host, n * sizeof(double));  // while the conversion runs
         CK(cudaMemcpyAsync(host, dtmp, n * sizeof(double), cudaMemcpyDeviceToHost, st));
         CK(cudaStreamSynchronize(st));
         return RVE_OK;
