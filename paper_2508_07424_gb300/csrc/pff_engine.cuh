@@ -40,7 +40,6 @@
 #include "pff_batch.cuh"
 #include "pff_common.cuh"
 #include "pff_functors.cuh"
-#include "pff_host.cuh"
 #include "pff_kernels.cuh"
 #include "pff_newton.cuh"
 
@@ -1179,7 +1178,7 @@ struct Engine : EngineBase {
     template <typename K> void prep_smem(K kernel, size_t bytes) {
         size_t &known = smem_set[(const void *)kernel];  // this handle's view: never above what is set
         if (known >= bytes) return;
-        CK(smem_raise(kernel, bytes));
+        CK(smem_raise((const void *)kernel, bytes));
         known = bytes;
     }
     // Events around one launch while timing is on (returns the end event to record after it).

@@ -1,11 +1,16 @@
-// Host-side helpers of the library that need neither a kernel nor a device.
+// Host-side helpers of the library: plain C++ that compiles without nvcc.
 #pragma once
 
+#include <cuda_runtime_api.h>
 #include <sys/mman.h>
 #include <unistd.h>
 
 #include <cstddef>
 #include <cstdint>
+#include <exception>
+#include <map>
+#include <mutex>
+#include <utility>
 
 #ifndef MADV_POPULATE_WRITE
 #define MADV_POPULATE_WRITE 23
@@ -24,6 +29,30 @@ inline void map_pages(void *p, size_t bytes) {
     if (!p || !bytes) return;
     const uintptr_t a = (uintptr_t)p & ~(page - 1), e = ((uintptr_t)p + bytes + page - 1) & ~(page - 1);
     (void)madvise((void *)a, e - a, MADV_POPULATE_WRITE);
+}
+
+// Opt a kernel in to `bytes` of dynamic shared memory on the current device. The attribute belongs to the
+// kernel, not to a handle, and one instance serves every line length, so it is only ever raised: a
+// handle of a smaller grid must not lower it under a larger one's launches. Throws nothing: entry points with
+// C linkage call it outside any handler.
+inline std::mutex g_smem_mu;
+inline std::map<std::pair<int, const void *>, size_t> g_smem_max;
+inline cudaError_t smem_raise(const void *kernel, size_t bytes) noexcept {
+    // up to 32 KB needs no opt-in: static shared memory (reduction scratch) adds to the dynamic size
+    if (bytes <= 32 * 1024) return cudaSuccess;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    try {
+        std::lock_guard<std::mutex> lk(g_smem_mu);
+        size_t &cur = g_smem_max[{dev, kernel}];
+        if (cur >= bytes) return cudaSuccess;
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        if (e == cudaSuccess) cur = bytes;
+        return e;
+    } catch (const std::exception &) {  // no memory for the entry, or the mutex failed
+        return cudaErrorMemoryAllocation;
+    }
 }
 
 }  // namespace pff

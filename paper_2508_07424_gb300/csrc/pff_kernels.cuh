@@ -16,34 +16,13 @@
 #pragma once
 
 #include <algorithm>
-#include <map>
-#include <mutex>
 #include <type_traits>
-#include <utility>
 
 #include "pff_common.cuh"
 #include "pff_fixed.cuh"
+#include "pff_host.cuh"
 
 namespace pff {
-
-// Opt a kernel in to `bytes` of dynamic shared memory on the current device. The attribute belongs to the
-// kernel, not to a handle, and one instance serves every line length, so it is only ever raised: a
-// handle of a smaller grid must not lower it under a larger one's launches.
-inline std::mutex g_smem_mu;
-inline std::map<std::pair<int, const void *>, size_t> g_smem_max;
-template <class K> inline cudaError_t smem_raise(K kernel, size_t bytes) {
-    // up to 32 KB needs no opt-in: static shared memory (reduction scratch) adds to the dynamic size
-    if (bytes <= 32 * 1024) return cudaSuccess;
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    std::lock_guard<std::mutex> lk(g_smem_mu);
-    size_t &cur = g_smem_max[{dev, (const void *)kernel}];
-    if (cur >= bytes) return cudaSuccess;
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e == cudaSuccess) cur = bytes;
-    return e;
-}
 
 enum { AX_FWD = 0, AX_INV = 1, AX_FWD_OP_INV = 2 };
 

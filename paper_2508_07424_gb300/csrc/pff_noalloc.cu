@@ -204,7 +204,7 @@ extern "C" int rve_dissipation_noalloc(int dim, const int n[3], double ell, int 
         if (cudaGetLastError() != cudaSuccess) return RVE_ECUDA;
     }
     auto launch = [&](auto kernel, dim3 grid, int threads, size_t sm, auto... args) -> cudaError_t {
-        const cudaError_t e = smem_raise(kernel, sm);
+        const cudaError_t e = smem_raise((const void *)kernel, sm);
         if (e != cudaSuccess) return e;
         kernel<<<grid, threads, sm, st>>>(args...);
         return cudaGetLastError();

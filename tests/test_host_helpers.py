@@ -14,7 +14,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 def host(tmp_path_factory):
     so = str(tmp_path_factory.mktemp("host") / "host_helpers.so")
     cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
-    subprocess.run(["g++", "-std=c++17", "-O2", "-fPIC", "-shared", "-I", os.path.join(cuda, "include"), "-o", so,
+    # -Bsymbolic: the stand-ins for CUDA calls are the library's own, whatever else the process has loaded
+    subprocess.run(["g++", "-std=c++17", "-O2", "-fPIC", "-shared", "-Wl,-Bsymbolic", "-I", os.path.join(cuda, "include"), "-o", so,
                     os.path.join(HERE, "host_helpers.cpp")], check=True)
     return C.CDLL(so)
 
@@ -35,3 +36,21 @@ def test_mapping_pages_refuses_without_harm(host):
     host.map_pages(C.c_void_p(at), C.c_size_t(0))
     host.map_pages(C.c_void_p(at), C.c_size_t(1 << 16))
     host.map_pages(C.c_void_p(1 << 44), C.c_size_t(1 << 16))
+
+
+def test_shared_memory_opt_in(host):
+    """Only ever raised, not asked for again, an error is passed on and not remembered, and no memory for the
+    table is an error code too: an exception would leave through an entry point with C linkage."""
+    calls, size = C.c_int(), C.c_size_t()
+
+    def raise_to(kernel, kb, no_memory=0):
+        e = host.smem_raise(C.c_size_t(kernel), C.c_size_t(kb * 1024), no_memory, C.byref(calls), C.byref(size))
+        return e, calls.value, size.value // 1024
+
+    assert raise_to(16, 32) == (0, 0, 0)
+    assert raise_to(16, 100, no_memory=1) == (2, 0, 0)  # cudaErrorMemoryAllocation
+    assert raise_to(16, 100) == (0, 1, 100)
+    assert raise_to(16, 60) == (0, 1, 100)
+    assert raise_to(16, 100, no_memory=1) == (0, 1, 100)
+    assert raise_to(32, 228) == (1, 2, 228)  # cudaErrorInvalidValue
+    assert raise_to(32, 200) == (0, 3, 200)
