@@ -38,8 +38,17 @@ METRIC = "FFT-PFF voxel-updates/s"
 # read.sum + dram__bytes_write.sum of the captured launch), keyed by (workload, precision, kernel
 # class). A kernel without a capture of its current code reports null; an entry is removed when
 # the kernel it describes changes.
-TRAFFIC = {}
-TRAFFIC_SOURCE = {}
+TRAFFIC = {
+    ("fibre_composite_512", "fp64", "projection_pass"): 6415360 + 0,
+    ("fibre_composite_512", "fp64", "cg_x_fwd"): 34676480 + 1280,
+    ("polycrystal_3d_128", "fp32r", "projection_pass"): 53531904 + 5502464,
+    ("polycrystal_3d_128", "fp32r", "cg_x_fwd"): 272255744 + 196799744,
+}
+_F64, _P32 = "profiles/fixed_point_passes_fibre512_fp64.md", "profiles/cg_passes_poly128cubed_fp32.md"
+TRAFFIC_SOURCE = {
+    k: f"ncu, one launch in an equilibrium solve with plain launches, cold caches ({_F64 if k[1] == 'fp64' else _P32})"
+    for k in TRAFFIC
+}
 
 
 def workload_desc(name=WORKLOAD):
@@ -334,11 +343,14 @@ def roofline_of(bd, precision, workload, hbm_peak, hbm_src, f64):
     c = cls[dom]
     traffic = TRAFFIC.get((workload, precision, dom))
     if precision == "fp64":
-        # The FFT work against the FP64 FMA rate of this part (measured live), which bounded it when it ran in
-        # FP64. The lines are transformed in 64-bit integers now, so the fraction may pass 1.
+        # The FFT work against the FP64 FMA rate of this part (measured live), which would bound it in FP64. The
+        # lines are transformed in 64-bit integers, so this is an equivalent rate and no utilisation of that pipe
+        # (25 % busy in the projection pass); it may pass 1.
         ach, peak = c["TFLOP_s"], f64["tflops"]
         roof = {"bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
                 "peak_source": "measured in this run (rve_fp64_fma_rate)",
+                "frac_is": "equivalent FP64 FFT rate over the FP64 FMA rate, not a utilisation: the lines are transformed in "
+                           "64-bit integers",
                 "per_launch": "5 L log2 L flops per transformed line (FFT work only; transformed in 64-bit fixed point)",
                 "hbm_GB_s": c["GB_s"], "hbm_frac": c["GB_s"] / hbm_peak}
     else:

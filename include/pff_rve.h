@@ -216,7 +216,13 @@ int effective_toughness(rve_handle h, double *g_eff);
 int effective_toughness_functional(rve_handle h, double *g_eff);
 
 /* Copy a device field to / from a host buffer of n doubles (see RVE_FIELD_*). Setting PHI, H or
- * FLUCT1 lets a caller inject a committed state; setting PHI also copies it to the trial field. */
+ * FLUCT1 lets a caller inject a committed state; setting PHI also copies it to the trial field.
+ * rve_get_field writes to the buffer by the copy alone: a call refused with RVE_EINVAL leaves it as it was.
+ *
+ * Range. The FP64 transforms run in 64-bit fixed point with a scale per line (pff_fixed.cuh): as accurate as
+ * FP64 ones relative to the line, values below 2^-1022 count as zero, and a line whose sum of moduli passes
+ * 2^1024 gives NaN although its single values may be finite (energies and norms are sums of squares, which
+ * underflow and overflow long before). A NaN or an infinity makes its line NaN and the solve RVE_EBREAKDOWN. */
 int rve_get_field(rve_handle h, int field, double *host, size_t n);
 int rve_set_field(rve_handle h, int field, const double *host, size_t n);
 int rve_get_scalars(rve_handle h, rve_scalars *s);

@@ -497,6 +497,11 @@ template <int K> struct axis_form_of {
     static constexpr bool TWO = K >= AXK_8T;
 };
 // FP32 lines of 16 to 128 points: 80 registers, 3 CTAs of 256 threads per SM (128^3 projection pass 49.4 -> 45.1 us).
+// The bound spills 40 to 68 bytes in every operator, which pays where there are more than two CTAs per SM and costs
+// where there are not. FP32R solves with the bound against without: 128^3 3 % (equilibrium) and 6 % (damage) faster,
+// 128x128x64 3.5 %, 64^3 1 and 2.6 %, 64x64x16 1.5 and 2.6 %; 128^2 and 64^2 1 to 1.7 % slower, 128x64x1 1 and 3 %;
+// 256^2 and more in 2D equal (those lines take the two-pass form). A second instance for small grids would double
+// the compilation of the column passes for those few percent.
 template <typename T, int K> __host__ __device__ constexpr int axis_min_blocks() { return sizeof(T) == 4 && K == AXK_16 ? 3 : 0; }
 
 // ---- x passes ------------------------------------------------------------------------------------
@@ -506,7 +511,9 @@ template <typename T, int K> __host__ __device__ constexpr int axis_min_blocks()
 // bounded for occupancy: 64 up to three components (the 512 CTAs of 256 threads of a 1024^2 pass fit the 608
 // slots in one wave instead of two, 43.6 -> 31.8 us per CG forward launch), 72 with six (the 2048 CTAs of
 // 128 threads of a 128^3 pass in two waves instead of three: CG forward 154 -> 131 us, inverse
-// 66 -> 59 us; 85 registers gain no wave and measured 5-10 % slower). FP64: two CTAs per SM.
+// 66 -> 59 us; 85 registers gain no wave and measured 5-10 % slower). FP64: two CTAs per SM. The rule goes by the
+// number of components; with it and the fixed-point residual passes the FP32R equilibrium is 1.02 to 1.40 times
+// as fast on all of 17 grids (2D 64^2 to 1024^2 and 1024x64, 3D 16^3 to 128^3, plates).
 template <typename T, int NC> __host__ __device__ constexpr int x_max_regs() { return sizeof(T) == 8 ? 128 : (NC <= 3 ? 64 : 72); }
 template <typename T> __host__ __device__ constexpr int x_mid_threads() { return sizeof(T) == 8 ? 256 : 512; }
 
@@ -515,13 +522,14 @@ template <typename T> __host__ __device__ constexpr int x_mid_threads() { return
 // small grids an FP64 pass is bound by the FP64 work of the few SMs that hold a CTA, so there a CTA
 // takes as few row pairs as give a whole warp, until there are two CTAs per SM (64^2 with the
 // split: 4 -> 32 CTAs, 66 -> 24 us per forward pass; FP32 passes gained nothing from it).
+constexpr int kSmCount = 152;  // GB300
 struct XShape { int threads, blocks, RP; };
 template <typename T> inline XShape x_shape(int nx, long long pairs) {
     constexpr bool fx = sizeof(T) == 8;
     const int unit = fx ? nx : nx / 4;  // FP64: columns, FP32: threads of a row pair
     const int full = fx ? 256 : 128;
     int RP = full / unit > 1 ? full / unit : 1;
-    while (RP > 1 && (RP > pairs || (fx && pairs / RP < 304 && RP / 2 * unit >= 32))) RP >>= 1;
+    while (RP > 1 && (RP > pairs || (fx && pairs / RP < 2 * kSmCount && RP / 2 * unit >= 32))) RP >>= 1;
     XShape x;
     x.RP = RP;
     x.blocks = (int)(pairs / RP);
