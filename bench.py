@@ -44,11 +44,8 @@ TRAFFIC = {
     ("polycrystal_3d_128", "fp32r", "projection_pass"): 53531904 + 5502464,
     ("polycrystal_3d_128", "fp32r", "cg_x_fwd"): 272255744 + 196799744,
 }
-_F64, _P32 = "profiles/fixed_point_passes_fibre512_fp64.md", "profiles/cg_passes_poly128cubed_fp32.md"
-TRAFFIC_SOURCE = {
-    k: f"ncu, one launch in an equilibrium solve with plain launches, cold caches ({_F64 if k[1] == 'fp64' else _P32})"
-    for k in TRAFFIC
-}
+TRAFFIC_SOURCE = {k: "ncu, one launch in an equilibrium solve with plain launches, cold caches (summaries in profiles/)"
+                  for k in TRAFFIC}
 
 
 def workload_desc(name=WORKLOAD):
